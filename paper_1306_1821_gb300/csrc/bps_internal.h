@@ -31,6 +31,10 @@ struct PassTable {
   void (*x_macc)(const Fields&, int region, int nch, cudaStream_t);    // acc += delta, mass-bin power
   void (*x_mmean)(const Fields&, int region, int nch, cudaStream_t);   // mass-bin power of acc
   void (*x_wpow)(const Fields&, int region, int nch, cudaStream_t);    // power-bin power of W
+  // one chain, mock field: W = IFFT_x(amp[|n|^2] FFT_x(W)), and dst = the z transform
+  // of the normals of stream (seed, 0, stage, 0)
+  void (*x_amp)(const Fields&, const float* amp, cudaStream_t);
+  void (*z_mock)(const Fields&, uint64_t seed, uint64_t stage, float2* dst, cudaStream_t);
   void (*y_fwd)(const Fields&, int buf, int nch, cudaStream_t);
   void (*y_inv)(const Fields&, int buf, int nch, cudaStream_t);
   void (*z_grad)(const Fields&, int region, int nch, cudaStream_t);

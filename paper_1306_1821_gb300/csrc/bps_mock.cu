@@ -26,108 +26,212 @@ constexpr double CHUNK_MEAN = 32.0;    // largest mean of one inversion chunk
 constexpr double LAMBDA_MAX = 4096.0;  // larger means give the out-of-range count 65536
 constexpr int MAX_STEPS = 200;         // bound of one chunk's inversion search
 
-// normals of stream (seed, 0, ST_MOCK_FIELD, 0): element i from block i/8, the
-// FP32 Box-Muller pair of word (i % 8)/2, cosine branch for even i
-__global__ void k_mock_normals(uint64_t seed, size_t n, float* out) {
-  const size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (q * 8 >= n) return;
-  P4 r = philox(q, 0, ST_MOCK_FIELD, 0, seed);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    float u1, u2;
-    u24pair(r.w[j], u1, u2);
-    const float rad = sqrtf(-2.f * logf(u1));
-    float sn, cs;
-    sincospif(2.f * u2, &sn, &cs);
-    if (q * 8 + 2 * j < n) out[q * 8 + 2 * j] = rad * cs;
-    if (q * 8 + 2 * j + 1 < n) out[q * 8 + 2 * j + 1] = rad * sn;
-  }
-}
-
-// W[ix][iy][iz] *= A[|n|^2] (padded half spectrum, rows of zp)
-__global__ void k_mock_amp(float2* W, int N, int zp, const double* amp) {
-  const long long H1 = N / 2 + 1, total = (long long)N * N * H1;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int iz = (int)(i % H1);
-    const long long row = i / H1;
-    const int iy = (int)(row % N), ix = (int)(row / N);
-    const int nx = ix <= N / 2 ? ix : ix - N, ny = iy <= N / 2 ? iy : iy - N;
-    const float a = (float)amp[nx * nx + ny * ny + iz * iz];
-    float2& v = W[row * zp + iz];
-    v.x *= a;
-    v.y *= a;
-  }
+// amplitudes A = sqrt(P / V_cell) of every |n|^2 (0 for k = 0): FP64, rounded to FP32
+__global__ void k_mock_amp(const double* __restrict__ P, int n, double vc, float* __restrict__ amp) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) amp[i] = i == 0 ? 0.f : __double2float_rn(__dsqrt_rn(__ddiv_rn(P[i], vc)));
 }
 
 struct Coef {
   double c[11];   // 1/j!, j = 0..10
 };
+constexpr Coef make_coef() {
+  Coef k{};
+  double fact = 1.0;
+  for (int j = 0; j <= 10; ++j) {
+    if (j > 0) fact *= j;
+    k.c[j] = 1.0 / fact;
+  }
+  return k;
+}
+__constant__ Coef c_coef = make_coef();
 
 // e^-mu for 0 <= mu <= 32: mu 2^-10 (exact), Taylor series of e^-x to degree
 // 10 by Horner's rule, then ten squarings (IEEE-exact operations only)
-__device__ __forceinline__ double exp_neg(double mu, const Coef& k) {
+__device__ __forceinline__ double exp_neg(double mu) {
   const double y = -__dmul_rn(mu, 0x1p-10);
-  double s = k.c[10];
+  double s = c_coef.c[10];
 #pragma unroll
-  for (int j = 9; j >= 0; --j) s = __dadd_rn(__dmul_rn(s, y), k.c[j]);
+  for (int j = 9; j >= 0; --j) s = __dadd_rn(__dmul_rn(s, y), c_coef.c[j]);
 #pragma unroll
   for (int q = 0; q < 10; ++q) s = __dmul_rn(s, s);
   return s;
 }
 
+// b and Nbar of every subsample, and their splits into two FP32 parts
 struct MockSub {
   double b[MAXS], nbar[MAXS];
+  float2 b2[MAXS], nbar2[MAXS];
 };
 
-// counts of subsample blockIdx.y: noise 0 Poisson(lambda) by chunked CDF
-// inversion, lambda = (R Nbar) max(0, 1 + b delta); noise 1 the Gaussian
-// noise model, round((R Nbar)(1 + b delta) + sqrt(R Nbar) z) clipped at 0
-__global__ void k_mock_counts(const float* __restrict__ delta, const float* __restrict__ R, long long nv,
-                              MockSub sub, Coef coef, int noise, uint64_t seed, int32_t* out) {
-  const int l = blockIdx.y;
-  const double b = sub.b[l], nbar = sub.nbar[l];
-  const float* Rl = R + (long long)l * nv;
-  int32_t* ol = out + (long long)l * nv;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double d = (double)delta[i];
-    const double rn = __dmul_rn((double)Rl[i], nbar);
-    double t = __dadd_rn(1.0, __dmul_rn(b, d));
-    if (noise == 0) {
-      t = fmax(0.0, t);
-      const double lam = __dmul_rn(rn, t);
-      if (!(lam <= LAMBDA_MAX)) {
-        ol[i] = 65536;
-        continue;
-      }
-      const double K = ceil(__ddiv_rn(lam, CHUNK_MEAN));
-      const double mu = K > 0.0 ? __ddiv_rn(lam, K) : 0.0;
-      const double e = exp_neg(mu, coef);
-      int total = 0;
-      const int nk = (int)K;
-      P4 r{};
-      for (int j = 0; j < nk; ++j) {
-        if ((j & 3) == 0) r = philox((uint64_t)i, (uint64_t)(j >> 2), ST_MOCK_COUNTS, (uint64_t)l, seed);
-        const double u = u52(r.w[j & 3]);
-        double p = e, F = e;
-        int k = 0;
-        while (u > F && k < MAX_STEPS) {
-          ++k;
-          p = __ddiv_rn(__dmul_rn(p, mu), (double)k);
-          F = __dadd_rn(F, p);
-        }
-        total += k;
-      }
-      ol[i] = total;
-    } else {
-      const double m = __dmul_rn(rn, t);
-      const P4 r = philox((uint64_t)i, 0, ST_MOCK_COUNTS, (uint64_t)l, seed);
-      const double u1 = u52(r.w[0]), u2 = u52(r.w[1]);
-      const double z = sqrt(-2.0 * log(u1)) * cos(__dmul_rn(2.0 * 3.141592653589793, u2));
-      const double x = __dadd_rn(m, __dmul_rn(__dsqrt_rn(rn), z));
-      const double c = floor(__dadd_rn(x, 0.5));
-      ol[i] = rn > 0.0 ? (int32_t)fmax(c, 0.0) : 0;
+// FP32 pairs (x + y, |y| <= half an ulp of x): about 46 significant bits from
+// FP32 arithmetic.  FP64 instructions, conversions included, issue at 1/64 of
+// the FP32 rate here, so the mock kernels decide in pairs and keep FP64 for
+// what the pairs cannot decide.
+__device__ __forceinline__ float2 pair_quick(float a, float b) {   // |a| >= |b| or a = 0
+  const float s = __fadd_rn(a, b);
+  return make_float2(s, __fsub_rn(b, __fsub_rn(s, a)));
+}
+__device__ __forceinline__ float2 pair_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+  return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z)));
+}
+__device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  return pair_quick(p, __fmaf_rn(a.x, b.y, __fmaf_rn(a.y, b.x, __fmaf_rn(a.x, b.x, -p))));
+}
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  const float2 s = pair_sum(a.x, b.x);
+  return pair_quick(s.x, __fadd_rn(s.y, __fadd_rn(a.y, b.y)));
+}
+
+// Inversion of the Poisson distribution function of mean mu (0 < mu <= 32) at u:
+// the smallest k with u <= F_k, in the FP64 operations that define the counts.
+__device__ __noinline__ int poisson_invert(double mu, double u) {
+  double p = exp_neg(mu), F = p;
+  int k = 0;
+  while (u > F && k < MAX_STEPS) {
+    ++k;
+    p = __ddiv_rn(__dmul_rn(p, mu), (double)k);
+    F = __dadd_rn(F, p);
+  }
+  return k;
+}
+
+// 1 / k and the width of the undecided band around F_k, in units of F_k
+struct ScreenTable {
+  float inv[MAX_STEPS + 8], tol[MAX_STEPS + 8];
+};
+constexpr ScreenTable make_screen_table() {
+  ScreenTable t{};
+  for (int k = 0; k < MAX_STEPS + 8; ++k) {
+    t.inv[k] = k == 0 ? 0.f : (float)(1.0 / (double)k);
+    t.tol[k] = (float)((k + 2) * 4e-7);
+  }
+  return t;
+}
+__constant__ ScreenTable c_screen = make_screen_table();
+
+// The same search in FP32 for the mean mu (an FP32 pair, off by less than 1e-10),
+// with a bound on how far its F_k can be from the FP64 one; -1 where u lies
+// within the bound of some F_k it meets, for the caller to decide in FP64.
+// Bound, in units of 2^-24: e^-mu is off by 5 (expf 4, the pair's second part
+// 1), each step of p by 4 (mu, 1 / k and two products) and each addition by 1,
+// so F_k is off by at most (5 + 5 k) 2^-24 < (k + 1) 3e-7 of itself; u is rounded
+// to FP32 (2^-24 of itself, and F is as large where it matters) from its upper
+// 32 bits (2.4e-10).  Taken as (k + 2) 4e-7 F + 1e-9, it leaves about 1e-6 (k + 2)
+// of the draws undecided.  The lanes of a warp walk through the same k together,
+// four steps between tests: the chain of a step is one product and one sum.
+__device__ __forceinline__ int poisson_screen(float2 mu, uint64_t w) {
+  float p = expf(-mu.x);
+  p = fmaf(-p, mu.y, p);
+  const float u = __fmul_rn(__uint2float_rn((uint32_t)(w >> 32)), 0x1p-32f);
+  float F = p;
+  int n = 0;
+  bool unsure = false;
+  for (int k = 0; k < MAX_STEPS; k += 4) {
+    float d = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      d = u - F;
+      unsure |= fabsf(d) <= fmaf(F, c_screen.tol[k + j], 1e-9f);
+      n += d > 0.f;
+      p *= mu.x * c_screen.inv[k + j + 1];
+      F += p;
+    }
+    if (d < 0.f || unsure) return unsure ? -1 : n;
+  }
+  return -1;
+}
+
+// The Poisson count of voxel i and subsample l with response r and field d by
+// definition: lambda = (r Nbar) max(0, 1 + b d), in ceil(lambda / 32) chunks of equal mean.
+__device__ __noinline__ int poisson_exact(float r, float d, double b, double nbar, long long i, int l, uint64_t seed) {
+  const double rn = __dmul_rn((double)r, nbar);
+  const double t = fmax(0.0, __dadd_rn(1.0, __dmul_rn(b, (double)d)));
+  const double lam = __dmul_rn(rn, t);
+  if (!(lam <= LAMBDA_MAX)) return 65536;
+  const double K = ceil(__ddiv_rn(lam, CHUNK_MEAN));
+  const double mu = K > 0.0 ? __ddiv_rn(lam, K) : 0.0;
+  const int nk = (int)K;
+  const float m = (float)mu;
+  const float2 m2 = make_float2(m, (float)(mu - (double)m));
+  int total = 0;
+  P4 w{};
+  for (int j = 0; j < nk; ++j) {
+    if ((j & 3) == 0) w = philox((uint64_t)i, (uint64_t)(j >> 2), ST_MOCK_COUNTS, (uint64_t)l, seed);
+    const uint64_t wj = (j & 3) == 0 ? w.w[0] : (j & 3) == 1 ? w.w[1] : (j & 3) == 2 ? w.w[2] : w.w[3];
+    int k = poisson_screen(m2, wj);
+    if (k < 0) k = poisson_invert(mu, u52(wj));
+    total += k;
+  }
+  return total;
+}
+
+// The same count without FP64 where FP32 pairs decide it: one chunk (lambda
+// safely below 32) of ordinary factors.  The pair for 1 + b d is off by less
+// than 2^-43 (1 + |b d|), that for lambda by less than 2^-42 r Nbar (1 + |b d|),
+// which is below 1e-10 for the factors let through.
+__device__ __noinline__ int poisson_count(float r, float d, float2 b, float2 nb, double b64, double nbar64, long long i,
+                                          int l, uint64_t seed) {
+  const float q = __fmul_rn(b.x, d);
+  const float2 bd = pair_quick(q, __fmaf_rn(b.y, d, __fmaf_rn(b.x, d, -q)));
+  const float2 t = pair_add(make_float2(1.f, 0.f), bd);
+  const float2 rn = pair_mul(make_float2(r, 0.f), nb);
+  if (r > 0.f && rn.x * (1.f + fabsf(q)) < 400.f) {   // false for NaN
+    if (t.x <= -1e-6f * (1.f + fabsf(q))) return 0;   // lambda = 0
+    float2 lam = pair_mul(rn, t);
+    if (lam.x < 0.f) lam = make_float2(0.f, 0.f);     // 1 + b d = 0 to within the pair's error
+    if (lam.x < 31.9f) {
+      const int k = poisson_screen(lam, philox((uint64_t)i, 0, ST_MOCK_COUNTS, (uint64_t)l, seed).w[0]);
+      if (k >= 0) return k;
+    }
+  }
+  return poisson_exact(r, d, b64, nbar64, i, l, seed);
+}
+
+// The paper's Gaussian noise: round((r Nbar)(1 + b d) + sqrt(r Nbar) z) clipped at 0.
+__device__ __forceinline__ int gauss_count(float r, float d, double b, double nbar, long long i, int l,
+                                           uint64_t seed) {
+  const double rn = __dmul_rn((double)r, nbar);
+  if (!(rn > 0.0)) return 0;
+  const double m = __dmul_rn(rn, __dadd_rn(1.0, __dmul_rn(b, (double)d)));
+  const P4 w = philox((uint64_t)i, 0, ST_MOCK_COUNTS, (uint64_t)l, seed);
+  const double u1 = u52(w.w[0]), u2 = u52(w.w[1]);
+  const double z = sqrt(-2.0 * log(u1)) * cos(__dmul_rn(2.0 * 3.141592653589793, u2));
+  const double x = __dadd_rn(m, __dmul_rn(__dsqrt_rn(rn), z));
+  return (int32_t)fmax(floor(__dadd_rn(x, 0.5)), 0.0);
+}
+
+// Counts of every subsample (noise 0: Poisson by inversion, noise 1: Gaussian),
+// one voxel per thread, the subsamples in the inner loop so that the field is
+// read once.  FP64 issue bounds any FP64 work here: 13.8 ms at 256^3 with six
+// subsamples with every voxel searched in FP64, 1.72 ms with lambda in FP64 and
+// the search in FP32 at the observed voxels only (FP64 pipe 77% busy), and
+// 0.55 ms with lambda in FP32 pairs as well: ALU and FMA pipes 35% and 29% busy,
+// the rest loads.  Four voxels per thread hold 124 registers and two blocks per
+// SM (0.92 ms); one response in flight per thread instead of four takes 0.70 ms.
+template <int NOISE>
+__global__ void __launch_bounds__(256, 4) k_mock_counts(const float* __restrict__ delta, const float* __restrict__ R,
+                                                        long long nv, int nsub, MockSub sub, uint64_t seed,
+                                                        int32_t* __restrict__ out) {
+  constexpr int G = 4;   // responses in flight per thread: most voxels only pass through
+  const long long i = blockIdx.x * 256LL + threadIdx.x;
+  if (i >= nv) return;
+  const float d = delta[i];
+  for (int l0 = 0; l0 < nsub; l0 += G) {
+    float r[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) r[g] = l0 + g < nsub ? R[(l0 + g) * nv + i] : 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const int l = l0 + g;
+      if (l >= nsub) break;
+      int c = 0;
+      if constexpr (NOISE) c = gauss_count(r[g], d, sub.b[l], sub.nbar[l], i, l, seed);
+      else if (!(r[g] == 0.f && isfinite(d)))   // lambda = 0 there
+        c = poisson_count(r[g], d, sub.b2[l], sub.nbar2[l], sub.b[l], sub.nbar[l], i, l, seed);
+      out[l * nv + i] = c;
     }
   }
 }
@@ -139,36 +243,124 @@ struct RespArgs {
 };
 
 // R[l][i] = [cos(theta_i) >= 1 - 2 f_sky and r_i <= r_max] * table_l(r_i),
-// the table sampled at r_j = j r_max / (n_r - 1) and interpolated linearly
-__global__ void k_mock_response(RespArgs a, const double* __restrict__ table, float* __restrict__ R) {
-  const long long nv = (long long)a.N * a.N * a.N;
-  const double nrm = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(a.ax, a.ax), __dmul_rn(a.ay, a.ay)),
-                                          __dmul_rn(a.az, a.az)));
-  const double ux = __ddiv_rn(a.ax, nrm), uy = __ddiv_rn(a.ay, nrm), uz = __ddiv_rn(a.az, nrm);
+// the table sampled at r_j = j r_max / (n_r - 1) and interpolated linearly.
+// V consecutive voxels of one z line per thread.  In half voxels the coordinates
+// are odd integers, so 4 r^2 = S is an exact integer in FP32, S = N^2 mod 8 never
+// holds (three odd squares are 3 mod 8) and r <= r_max is S < N^2; the FP32
+// cosine is off by less than 1e-6 and decides the cap outside a margin of 1e-5.
+// Values are computed as FP32 pairs (t = sqrt(S) (n_r - 1) / N, table entries split
+// in two), off by less than 2^-41 of the larger table entry and 2^-43 t of the step
+// between the two, and kept where that cannot change their rounding to FP32; the rest takes the FP64 steps that define
+// the response.  With every voxel in FP64 the kernel was bound by FP64 issue: 2.59
+// ms at 256^3 with six subsamples, 0.76 ms with FP64 inside the survey only, now
+// 0.146 ms.
+__device__ __noinline__ float response_exact(const RespArgs& a, int ix, int iy, int iz, double ux, double uy, double uz,
+                                             const double* __restrict__ tl) {
   const double nr1 = (double)(a.n_r - 1);
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int iz = (int)(i % a.N);
+  const double x = __dsub_rn(__dmul_rn((double)ix + 0.5, a.dx), a.half_box);
+  const double y = __dsub_rn(__dmul_rn((double)iy + 0.5, a.dx), a.half_box);
+  const double z = __dsub_rn(__dmul_rn((double)iz + 0.5, a.dx), a.half_box);
+  const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)));
+  const double proj = __dadd_rn(__dadd_rn(__dmul_rn(ux, x), __dmul_rn(uy, y)), __dmul_rn(uz, z));
+  const double cos_t = r > 0.0 ? __ddiv_rn(proj, r) : 1.0;
+  if (!(cos_t >= a.thr_cos && r <= a.r_max)) return 0.f;
+  const double t = fmin(__dmul_rn(__ddiv_rn(r, a.r_max), nr1), nr1);
+  const double jf = fmin(floor(t), nr1 - 1.0);
+  const int j = (int)jf;
+  const double w = __dsub_rn(t, jf);
+  return __double2float_rn(__dadd_rn(__dmul_rn(tl[j], __dsub_rn(1.0, w)), __dmul_rn(tl[j + 1], w)));
+}
+
+// the table as FP32 pairs, and the unit axis
+__global__ void k_mock_table(RespArgs a, const double* __restrict__ table, long long n, float2* __restrict__ out,
+                             double* __restrict__ axis) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i == 0) {
+    const double nrm = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(a.ax, a.ax), __dmul_rn(a.ay, a.ay)),
+                                            __dmul_rn(a.az, a.az)));
+    axis[0] = __ddiv_rn(a.ax, nrm);
+    axis[1] = __ddiv_rn(a.ay, nrm);
+    axis[2] = __ddiv_rn(a.az, nrm);
+  }
+  if (i >= n) return;
+  const float h = (float)table[i];
+  out[i] = make_float2(h, (float)(table[i] - (double)h));
+}
+
+template <int V>
+__global__ void __launch_bounds__(256, 4) k_mock_response(RespArgs a, float2 c2, const double* __restrict__ axis,
+                                                          const double* __restrict__ table,
+                                                          const float2* __restrict__ table2, float* __restrict__ R) {
+  const float uxf = (float)axis[0], uyf = (float)axis[1], uzf = (float)axis[2];
+  const float cos_out = (float)a.thr_cos - 1e-5f, cos_in = (float)a.thr_cos + 1e-5f;
+  const float jmax = (float)(a.n_r - 2);
+  const long long nv = (long long)a.N * a.N * a.N;
+  const long long i = (blockIdx.x * 256LL + threadIdx.x) * V;
+  if (i < nv) {
+    const int iz0 = (int)(i % a.N);
     const int iy = (int)((i / a.N) % a.N);
     const int ix = (int)(i / ((long long)a.N * a.N));
-    const double x = __dsub_rn(__dmul_rn((double)ix + 0.5, a.dx), a.half_box);
-    const double y = __dsub_rn(__dmul_rn((double)iy + 0.5, a.dx), a.half_box);
-    const double z = __dsub_rn(__dmul_rn((double)iz + 0.5, a.dx), a.half_box);
-    const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)));
-    const double proj = __dadd_rn(__dadd_rn(__dmul_rn(ux, x), __dmul_rn(uy, y)), __dmul_rn(uz, z));
-    const double cos_t = r > 0.0 ? __ddiv_rn(proj, r) : 1.0;
-    const bool inside = cos_t >= a.thr_cos && r <= a.r_max;
-    const double t = fmin(__dmul_rn(__ddiv_rn(r, a.r_max), nr1), nr1);
-    const int j = (int)fmin(floor(t), nr1 - 1.0);
-    const double w = __dsub_rn(t, (double)j);
-    const double omw = __dsub_rn(1.0, w);
+    const int x = 2 * ix + 1 - a.N, y = 2 * iy + 1 - a.N;
+    const float pxy = uxf * (float)x + uyf * (float)y;
+    int state[V];            // 0 outside, 1 inside, 2 undecided
+    int jt[V];
+    float2 w[V];
+    bool any = false;
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+      const int z = 2 * (iz0 + e) + 1 - a.N;
+      const int S = x * x + y * y + z * z;
+      const float Sf = (float)S;
+      const float cf = (pxy + uzf * (float)z) * rsqrtf(Sf);
+      state[e] = 0;
+      jt[e] = 0;
+      w[e] = make_float2(0.f, 0.f);
+      if (S >= a.N * a.N || cf < cos_out) continue;
+      any = true;
+      if (!(cf > cos_in)) {
+        state[e] = 2;
+        continue;
+      }
+      state[e] = 1;
+      const float s = sqrtf(Sf);
+      const float2 s2 = pair_quick(s, __fdividef(__fmaf_rn(-s, s, Sf), 2.f * s));
+      const float2 t = pair_mul(s2, c2);
+      const float j = fminf(fmaxf(floorf(t.x), 0.f), jmax);
+      jt[e] = (int)j;
+      w[e] = pair_sum(t.x - j, t.y);   // t.x - j is exact
+    }
     for (int l = 0; l < a.n_sub; ++l) {
-      const double* tl = table + (long long)l * a.n_r;
-      const double f = __dadd_rn(__dmul_rn(tl[j], omw), __dmul_rn(tl[j + 1], w));
-      R[(long long)l * nv + i] = inside ? __double2float_rn(f) : 0.f;
+      float v[V];
+#pragma unroll
+      for (int e = 0; e < V; ++e) v[e] = 0.f;
+      if (any) {
+        const double* tl = table + (long long)l * a.n_r;
+        const float2* tl2 = table2 + (long long)l * a.n_r;
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          if (state[e] == 0) continue;
+          bool ok = false;
+          if (state[e] == 1) {
+            const float2 t0 = __ldg(tl2 + jt[e]), t1 = __ldg(tl2 + jt[e] + 1);
+            const float2 f = pair_add(t0, pair_mul(w[e], pair_add(t1, make_float2(-t0.x, -t0.y))));
+            const float big = fmaxf(t0.x, t1.x);
+            const float tol = 0x1p-41f * big + 0x1p-43f * ((float)(jt[e] + 1) * fabsf(t1.x - t0.x));
+            // far from FP32's smallest and largest values, and rounded the same anywhere within tol
+            ok = (big == 0.f || (big > 1e-20f && big < 1e30f)) && __fadd_rn(f.x, f.y + tol) == f.x &&
+                 __fadd_rn(f.x, f.y - tol) == f.x;
+            v[e] = f.x;
+          }
+          if (!ok) v[e] = response_exact(a, ix, iy, iz0 + e, axis[0], axis[1], axis[2], tl);
+        }
+      }
+      float* Rl = R + (long long)l * nv + i;
+      if constexpr (V == 4) *reinterpret_cast<float4*>(Rl) = make_float4(v[0], v[1], v[2], v[3]);
+      else *Rl = v[0];
     }
   }
 }
+
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 // ---------------------------------------------------------------- host: Schechter tables
 // Gauss-Legendre nodes and weights on [-1, 1] (Newton iteration on P_n from
@@ -298,33 +490,30 @@ bps_status mock_field(const MockView& v, uint64_t seed, const double* P_n2, floa
   const int N = v.N;
   const size_t nt = (size_t)3 * (N / 2) * (N / 2) + 1;
   const double vc = std::pow(v.box / N, 3);
-  std::vector<double> amp(nt);
-  amp[0] = 0.0;
-  for (size_t i = 1; i < nt; ++i) {
-    if (!(P_n2[i] >= 0.0) || !std::isfinite(P_n2[i])) {
+  const std::vector<double> P(P_n2, P_n2 + nt);   // pageable: the copy below has left it when it returns
+  for (size_t i = 1; i < nt; ++i)
+    if (!(P[i] >= 0.0) || !std::isfinite(P[i])) {
       set_last_error("bps_mock_field: the spectrum must be finite and non-negative");
       return BPS_EINVAL;
     }
-    amp[i] = std::sqrt(P_n2[i] / vc);
-  }
-  double* damp = nullptr;
-  bps_status st = v.get_scratch(nt * sizeof(double), (void**)&damp);
+  double* dP = nullptr;   // the spectrum, then the FP32 amplitudes
+  bps_status st = v.get_scratch(nt * (sizeof(double) + sizeof(float)), (void**)&dP);
   if (st != BPS_OK) return st;
+  float* damp = reinterpret_cast<float*>(dP + nt);
   cudaStream_t s = v.stream;
-  if (cudaMemcpyAsync(damp, amp.data(), nt * sizeof(double), cudaMemcpyHostToDevice, s) != cudaSuccess) {
-    set_last_error("bps_mock_field: copy of the amplitude table failed");
+  if (cudaMemcpyAsync(dP, P.data(), nt * sizeof(double), cudaMemcpyHostToDevice, s) != cudaSuccess) {
+    set_last_error("bps_mock_field: copy of the spectrum failed");
     return BPS_ECUDA;
   }
-  const size_t nv = (size_t)N * N * N;
-  k_mock_normals<<<(unsigned)((nv / 8 + 255) / 256), 256, 0, s>>>(seed, nv, delta_dev);
-  v.pt->z_r2c(*v.f, delta_dev, v.f->W, s);
+  // the normals are drawn inside the first z pass, and the amplitudes applied
+  // between the two x transforms of one x pass
+  k_mock_amp<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(dP, (int)nt, vc, damp);
+  v.pt->z_mock(*v.f, seed, ST_MOCK_FIELD, v.f->W, s);
   v.pt->y_fwd(*v.f, BUF_W, 1, s);
-  v.pt->x_fwd(*v.f, BUF_W, v.f->W, 1, s);
-  k_mock_amp<<<v.n_sm * 8, 256, 0, s>>>(v.f->W, N, v.zp, damp);
-  v.pt->x_inv(*v.f, BUF_W, v.f->W, 1, s);
+  v.pt->x_amp(*v.f, damp, s);
   v.pt->y_inv(*v.f, BUF_W, 1, s);
   v.pt->z_c2r(*v.f, v.f->W, delta_dev, s);
-  *v.launches += 8;
+  *v.launches += 6;
   if (cudaGetLastError() != cudaSuccess) {
     set_last_error("bps_mock_field: kernel launch failed");
     return BPS_ECUDA;
@@ -342,16 +531,19 @@ bps_status mock_counts(const MockView& v, uint64_t seed, const float* delta_dev,
     }
     sub.b[l] = b[l];
     sub.nbar[l] = nbar[l];
-  }
-  Coef coef;
-  double fact = 1.0;
-  for (int j = 0; j <= 10; ++j) {
-    if (j > 0) fact *= j;
-    coef.c[j] = 1.0 / fact;
+    auto split = [](double x) {
+      const float h = (float)x;
+      return make_float2(h, (float)(x - (double)h));
+    };
+    sub.b2[l] = split(b[l]);
+    sub.nbar2[l] = split(nbar[l]);
   }
   const long long nv = (long long)v.N * v.N * v.N;
-  k_mock_counts<<<dim3(v.n_sm * 8, v.n_sub), 256, 0, v.stream>>>(delta_dev, R_dev, nv, sub, coef, noise, seed,
-                                                                  counts_dev);
+  // one block per 256 voxels: the hardware's block order balances the observed
+  // region, which a fixed stride over few blocks leaves to some of them
+  const unsigned blocks = (unsigned)((nv + 255) / 256);
+  if (noise == 0) k_mock_counts<0><<<blocks, 256, 0, v.stream>>>(delta_dev, R_dev, nv, v.n_sub, sub, seed, counts_dev);
+  else k_mock_counts<1><<<blocks, 256, 0, v.stream>>>(delta_dev, R_dev, nv, v.n_sub, sub, seed, counts_dev);
   *v.launches += 1;
   if (cudaGetLastError() != cudaSuccess) {
     set_last_error("bps_mock_counts: kernel launch failed");
@@ -374,7 +566,7 @@ bps_status mock_response(const MockView& v, double f_sky, const double* axis, in
       return BPS_EINVAL;
     }
   double* dt = nullptr;
-  bps_status st = v.get_scratch(tn * sizeof(double), (void**)&dt);
+  bps_status st = v.get_scratch((tn + 3) * sizeof(double) + tn * sizeof(float2), (void**)&dt);
   if (st != BPS_OK) return st;
   if (cudaMemcpyAsync(dt, table, tn * sizeof(double), cudaMemcpyHostToDevice, v.stream) != cudaSuccess) {
     set_last_error("bps_mock_response: copy of the selection table failed");
@@ -391,8 +583,18 @@ bps_status mock_response(const MockView& v, double f_sky, const double* axis, in
   a.ax = axis[0];
   a.ay = axis[1];
   a.az = axis[2];
-  k_mock_response<<<v.n_sm * 8, 256, 0, v.stream>>>(a, dt, R_dev);
-  *v.launches += 1;
+  double* axis_dev = dt + tn;
+  float2* dt2 = reinterpret_cast<float2*>(dt + tn + 3);
+  k_mock_table<<<(unsigned)((tn + 255) / 256), 256, 0, v.stream>>>(a, dt, (long long)tn, dt2, axis_dev);
+  const double c = (double)(n_r - 1) / (double)v.N;
+  const float2 c2 = make_float2((float)c, (float)(c - (double)(float)c));
+  const long long nv = (long long)v.N * v.N * v.N;
+  // 16-byte stores where R starts on a 16-byte boundary (every subsample then
+  // does: N^3 is a multiple of 4); one block per 1024 voxels, so that the
+  // hardware's block order balances the observed region
+  if (aligned16(R_dev)) k_mock_response<4><<<(unsigned)((nv / 4 + 255) / 256), 256, 0, v.stream>>>(a, c2, axis_dev, dt, dt2, R_dev);
+  else k_mock_response<1><<<(unsigned)((nv + 255) / 256), 256, 0, v.stream>>>(a, c2, axis_dev, dt, dt2, R_dev);
+  *v.launches += 2;
   if (cudaGetLastError() != cudaSuccess) {
     set_last_error("bps_mock_response: kernel launch failed");
     return BPS_ECUDA;

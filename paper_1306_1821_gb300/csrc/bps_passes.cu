@@ -32,7 +32,8 @@ enum XMode {
   X_MACC,       // acc += delta; per mass-bin sum w |delta|^2
   X_MMEAN,      // per mass-bin sum w |acc|^2
   X_WPOW,       // per-bin sum w |W|^2 (the power of whatever W holds)
-  X_LEAPG       // X_LEAP of the first step, also reducing g^T M^-1 g of the force it applies
+  X_LEAPG,      // X_LEAP of the first step, also reducing g^T M^-1 g of the force it applies
+  X_AMP         // W = IFFT_x(A(|n|^2) FFT_x(W))     (mock field: amplitudes between the transforms)
 };
 
 enum ZMode { Z_GRAD = 0, Z_NOISE, Z_R2C, Z_C2R, Z_SUMS };
@@ -45,6 +46,7 @@ struct XArgs {
   float2* dst;
   int first;
   int region;    // offset (doubles) of this launch's partial sums in Fields::part
+  const float* amp = nullptr;   // X_AMP: amplitude of every |n|^2
 };
 
 struct ZArgs {
@@ -57,6 +59,9 @@ struct ZArgs {
   // Z_C2R with mom: instead of writing delta, add delta and delta^2 to the
   // running sums mom[0..N^3) and mom[N^3..2 N^3) (FP64; posterior moments)
   double* mom = nullptr;
+  // Z_NOISE with a stage: the normals of stream (seed, 0, stage, 0) into dst
+  // instead of the move's momentum into the momentum spectrum
+  uint64_t stage = 0;
 };
 
 // ------------------------------------------------------------------ x pass helpers
@@ -183,7 +188,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
 
   // ---------------- modes that start from a spatial-x tile: forward transform
   if constexpr (MODE == X_INIT || MODE == X_LEAP || MODE == X_LEAPG || MODE == X_FINAL || MODE == X_FWD ||
-                MODE == X_GRAD || MODE == X_JGRAD) {
+                MODE == X_GRAD || MODE == X_JGRAD || MODE == X_AMP) {
     const float2* in = (MODE == X_INIT) ? fp.ph : (MODE == X_FWD) ? buf_ptr(fp, xa.src_buf) : fp.W;
     // X_FWD with no destination writes the current state buffer
     if (ja < R1) {
@@ -360,6 +365,23 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
     }
     double sP = block_sum2<NT>(eP, reinterpret_cast<float*>(s_red));
     if (t == 0) fp.part[xa.region + blockIdx.x] = sP;
+    return;
+  }
+
+  if constexpr (MODE == X_AMP) {
+    if (act) {
+#pragma unroll
+      for (int d = 0; d < R1; ++d) {
+        const int nx = sgn_n<N>(jc + R2 * d);
+        const float a = __ldg(xa.amp + nx * nx + n2yz);
+        v[d] = make_float2(__fmul_rn(v[d].x, a), __fmul_rn(v[d].y, a));   // rounded here: no FMA with the transform
+      }
+    }
+    fft2<N, R2, R1, INV, MAP_COL, F, TwSquare<N>::value>(v, s_ex, s_tw, t);
+    if (ja < R1) {
+#pragma unroll
+      for (int b = 0; b < R2; ++b) fp.W[colo + (long long)(ja + R1 * b) * T.rs] = v[b];
+    }
     return;
   }
 
@@ -1031,11 +1053,11 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
   } else {
     float* sr = reinterpret_cast<float*>(s_buf);
     if constexpr (MODE == Z_NOISE) {
-      const unsigned long long it = ds->iteration;
-      const uint64_t key = ds->seed;
+      const unsigned long long it = za.stage ? 0 : ds->iteration;
+      const uint64_t key = za.stage ? za.seed : ds->seed, stage = za.stage ? za.stage : (uint64_t)ST_MOMENTUM;
       const unsigned long long blk0 = (unsigned long long)(L0 * N) / 8;
       for (int q = t; q < LINES * N / 8; q += NTZ) {
-        P4 r = philox(blk0 + q, it, ST_MOMENTUM, 0, key);
+        P4 r = philox(blk0 + q, it, stage, 0, key);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           float u1, u2;
@@ -1189,7 +1211,7 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
     const int f = t / R2, c = t % R2;
     const int lane = t & 31;
     const int src = lane - c + (R2 - c) % R2;
-    float2* dst = (MODE == Z_GRAD) ? fp.W : (MODE == Z_NOISE) ? fp.ph : za.dst;
+    float2* dst = (MODE == Z_GRAD) ? fp.W : (MODE == Z_NOISE) ? (za.stage ? za.dst : fp.ph) : za.dst;
     float2* da = dst + (L0 + 2 * f) * ZP;
     float2* db = da + ZP;
 #pragma unroll
@@ -1656,6 +1678,8 @@ static PassTable make_table() {
   T.z_grad_lp[2] = [](const Fields& f, int region, int n, cudaStream_t s) { L::template z<Z_GRAD, 16>(f, ZArgs{nullptr, nullptr, nullptr, nullptr, region, 0}, n, s); };
   for (int i = 0; i < 3; ++i) T.z_lp_tiles[i] = N * N / (2 * (4 << i));
   T.z_noise = [](const Fields& f, int n, cudaStream_t s) { L::template z<Z_NOISE>(f, ZArgs{nullptr, nullptr, nullptr, nullptr, -1, 0}, n, s); };
+  T.x_amp = [](const Fields& f, const float* amp, cudaStream_t s) { L::template x<X_AMP>(f, XArgs{-1, nullptr, 0, -1, amp}, 1, s); };
+  T.z_mock = [](const Fields& f, uint64_t seed, uint64_t stage, float2* dst, cudaStream_t s) { L::template z<Z_NOISE>(f, ZArgs{nullptr, dst, nullptr, nullptr, -1, seed, nullptr, stage}, 1, s); };
   T.z_r2c = [](const Fields& f, const float* rin, float2* dst, cudaStream_t s) { L::template z<Z_R2C>(f, ZArgs{nullptr, dst, rin, nullptr, -1, 0}, 1, s); };
   T.z_c2r = [](const Fields& f, const float2* src, float* rout, cudaStream_t s) { L::template z<Z_C2R>(f, ZArgs{src, nullptr, nullptr, rout, -1, 0}, 1, s); };
   T.z_mom = [](const Fields& f, double* mom, cudaStream_t s) { L::template z<Z_C2R>(f, ZArgs{f.W, nullptr, nullptr, nullptr, -1, 0, mom}, 1, s); };
