@@ -499,7 +499,7 @@ bps_status bps_posterior_read(bps_ctx* ctx, double* mean_dev, double* var_dev, d
                               double* param_cov, uint64_t* n_samples);
 
 /* Self-test of failure detection.  Every device wait of the library (the bulk
- * tile copies of the z and fused y/z passes complete on shared-memory
+ * tile copies of the z passes and the staged x passes complete on shared-memory
  * mbarriers) is bounded: after 2 s the block gives up, records the timeout in
  * the chain's status word and exits, and the next call that reads the status
  * returns BPS_ETIMEOUT with the context still usable.  This call runs that

@@ -985,7 +985,7 @@ bps_status create_group(int grid_n, const std::vector<double>& box, const std::v
   // fused y^-1 / z / y stage where the grid has one; BPS_FUSED_YZ=0 keeps the three passes
   {
     const char* e = std::getenv("BPS_FUSED_YZ");
-    if (!(e && std::atoi(e) == 0) && !yz_table(grid_n, &ctx->yz)) ctx->yz = YzEntry{};
+    if (!(e && std::atoi(e) == 0) && !yz_table(grid_n, B, ctx->n_sm, &ctx->yz)) ctx->yz = YzEntry{};
   }
   ctx->part_stride = std::max(std::max(std::max(pt.x_tiles, pt.z_tiles), pt.z_lp_tiles[0]), ctx->rebuild_blocks);
   ctx->part_stride = std::max(ctx->part_stride, ctx->yz.tiles);

@@ -77,7 +77,7 @@ struct YzEntry {
   void (*run)(const Fields&, int region, int nch, cudaStream_t) = nullptr;
   int tiles = 0;
 };
-bool yz_table(int N, YzEntry* out);
+bool yz_table(int N, int nch, int n_sm, YzEntry* out);
 void launch_rebuild(const Fields& fp, long long nv, int region, int blocks, int nch, cudaStream_t s);
 // Data check of one subsample; with `span` (N a multiple of 32) it also widens
 // the per-line support of R > 0 (Fields::span encoding).

@@ -1,105 +1,96 @@
-// Fused y^-1 / z / y stage of the force evaluation (Eq. Wiener_Posterior_force):
-// one CTA (or one thread-block cluster) per x plane of the work spectrum
-// W(x, ky, kz).
+// Fused y^-1 / z / y stage of the force evaluation (Eq. Wiener_Posterior_force) on
+// grids whose x plane of the work spectrum W(x, ky, kz) fits one block's shared
+// memory: one block per plane, W read and written once (2 S_c + 2 S_r of HBM
+// traffic where the three separate passes take 6 S_c + 2 S_r).
 //
-// The three separate passes (inverse y transform, z pass with C2R, local force
-// and R2C, forward y transform) each read and write all of W: 6 S_c + 2 S_r of
-// HBM traffic.  Here a plane (N rows ky, ZP columns kz) is held in shared
-// memory, split over a cluster of CL CTAs when it does not fit one (CTA r
-// holds rows [r M, (r+1) M), M = N / CL), and is read and written once:
-// 2 S_c + 2 S_r.
+// What bounds it is the shared-memory pipe and the latency of its phases, so the
+// plane makes few trips and few barriers:
+//   - the first half of the inverse y transform reads W from global memory and the
+//     second half of the forward one writes it, both straight from registers;
+//   - the y transforms exchange in place.  With N = B A, the inverse reads
+//     x[j + A b], transforms over b and leaves t[j][c] in row j + A c; its second
+//     half transforms rows j + A c over j and leaves y = c + B d in row d + A c.
+//     The forward transform walks back the same way (first over d within the rows
+//     d + A c, then over c), so it ends in natural order, and neither needs a
+//     second buffer: one block barrier between the halves of each;
+//   - a warp owns eight consecutive z lines (four pairs, each one complex
+//     transform) from C2R through the local force to R2C: the exchanges go through
+//     the pair's own two rows with warp barriers only, and a warp whose lines
+//     carry no survey data writes zeros.
+// Rows are SP = ZP + 1 (odd) complex apart and the exchange within a pair is
+// swizzled (zpos), which keeps the 8-byte accesses of a half warp on distinct banks.
 //
-// With CL > 1 the y transforms are split radix-CL across the cluster (App. C.1
-// transform, length N = CL * M):
-//   inverse: out[CL m + r] = IFFT_M(b_r)[m],
-//            b_r[i] = e^{+2 pi i i r / N} sum_h in[i + M h] e^{+2 pi i h r / CL}
-//   forward: out[i + M r] = sum_r' e^{-2 pi i i r' / N} e^{-2 pi i r r' / CL} F_r'[i],
-//            F_r' = FFT_M of the rows y = CL m + r' held by CTA r'
-// so CTA r combines the CL row blocks of the cluster through distributed
-// shared memory, transforms its block along y (length M), and then holds the
-// complete z lines y = CL m + r, on which the z work runs locally.  The table
-// below builds the single-CTA form (CL = 1) for grids whose plane fits, where
-// it is faster than the three passes; the 256^3 plane would need a cluster, and
-// the cluster form measured slower than the passes there.
-#include <cooperative_groups.h>
-
+// Measured per launch under ncu against the form with a block-wide exchange buffer
+// (256 threads or fewer, 151 registers, 18% of the warp slots): 128^3 20.7 -> 14.4 us;
+// 32 chains of 96^3 162 -> 118 us, of 64^3 54 -> 34 us, of 32^3 10.8 -> 10.4 us.  At 96^3
+// the shared-memory pipe is 64-69% busy, with 40% of the warp slots filled.
 #include "bps_internal.h"
 #include "bps_passes.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace bps {
 namespace {
 
-template <int N, int CL>
+template <int N, int NWARPS>
 struct YZ {
-  static constexpr int M = N / CL;                       // rows per CTA
-  static constexpr int ZP = Cfg<N>::ZP, H = N / 2;
-  static constexpr int LP = 16;                          // z line pairs per round
-  static constexpr int R1 = Cfg<N>::R1, R2 = Cfg<N>::R2, RMAX = Cfg<N>::RMAX;      // z transform split
-  static constexpr int NT = LP * RMAX;                   // threads
-  static constexpr int MR1 = Cfg<M>::R1, MR2 = Cfg<M>::R2, MRMAX = Cfg<M>::RMAX;   // y transform split
-  static constexpr int FC = NT / MRMAX;                  // columns per y-transform round
-  static constexpr int GROUPS = (ZP + FC - 1) / FC;
-  static constexpr int ROUNDS = M / (2 * LP);            // z rounds
-  static constexpr int E = M * ZP;                       // elements of the block
-  static constexpr int CHUNK = (E + 2 * NT - 1) / (2 * NT);   // per-thread elements per combine chunk
-  static constexpr size_t BLK = (size_t)E * sizeof(float2);
-  static constexpr size_t EXC = (size_t)M * FC * sizeof(float2);
-  static constexpr size_t EXZ = (size_t)LP * (N + RMAX) * sizeof(float2);
-  static constexpr size_t EX = EXC > EXZ ? EXC : EXZ;
-  static constexpr size_t OFF_EX = BLK;
-  static constexpr size_t OFF_TWN = OFF_EX + EX;
-  static constexpr size_t OFF_TWM = OFF_TWN + (size_t)N * sizeof(float2);
-  static constexpr size_t OFF_RED = OFF_TWM + (size_t)M * sizeof(float2);
-  static constexpr size_t OFF_SPAN = OFF_RED + 32 * sizeof(double);      // lo[M], hi[M]
-  static constexpr size_t OFF_BAR = OFF_SPAN + (size_t)2 * M * sizeof(int);
-  static constexpr size_t BYTES = OFF_BAR + sizeof(uint64_t);
-  static_assert(N % CL == 0 && M % (2 * LP) == 0, "bad cluster split");
-  static_assert(NT % MRMAX == 0, "bad column split");
-  static_assert(EX >= (size_t)LP * N * sizeof(float2), "split buffer does not fit");
-  static_assert(BLK % 16 == 0, "bulk copy size");
+  static constexpr int B = Cfg<N>::R1, A = Cfg<N>::R2;   // N = B A, B >= A
+  static constexpr int ZP = Cfg<N>::ZP, H = N / 2, COLS = H + 1;
+  static constexpr int SP = ZP + 1;                      // row pitch in shared memory (complex)
+  static constexpr int T1 = A * COLS, T2 = B * COLS;     // tasks of the two halves of a y transform
+  static constexpr int PAIRS = 4, LINES = 2 * PAIRS;     // z lines of one warp unit
+  static constexpr int UNITS = N / LINES;
+  static constexpr int NW = NWARPS;
+  static constexpr int NT = 32 * NW;
+  static constexpr int ZT = PAIRS * B, ZR = (ZT + 31) / 32;   // second-half z tasks of a unit, rounds of them
+  static constexpr size_t OFF_TW = (size_t)N * SP * sizeof(float2);
+  static constexpr size_t OFF_TA = OFF_TW + (size_t)N * sizeof(float2);   // W^(a c) at c A + a
+  static constexpr size_t OFF_TB = OFF_TA + (size_t)N * sizeof(float2);   // W^(c e) at e B + c
+  static constexpr size_t BYTES = OFF_TB + (size_t)N * sizeof(float2);
+  static_assert(PAIRS * A <= 32, "a unit's first z half is one round");
+  static_assert(SP % 2 == 1 && UNITS * LINES == N , "layout");
+  // blocks per SM that the registers allow without spills
+  static constexpr int MIN_BLOCKS = 65536 / (NT * (N == 96 ? 73 : 80)) > 0 ? 65536 / (NT * (N == 96 ? 73 : 80)) : 1;
 };
 
-// v * exp(DIR 2 pi i k / CL), CL in {1, 2, 4}
-template <int CL, int DIR>
-__device__ __forceinline__ float2 root_cl(float2 v, int k) {
-  k %= CL;
-  if (k == 0) return v;
-  if (CL == 2 || k == 2) return make_float2(-v.x, -v.y);
-  return k == 1 ? mul_i<DIR>(v) : mul_i<-DIR>(v);
+// Slot (c, j), c < B, j < A, of the exchange of pair f: in [0, H) in the pair's
+// first row, in [H, N) in its second.
+template <int N>
+__device__ __forceinline__ int zpos(int c, int j, int f) {
+  constexpr int A = Cfg<N>::R2;
+  const int s = A == 8 ? (c ^ (c >> 3)) & 7 : ((c >> 2) | ((f & 1) << 1)) & (A - 1);
+  return c * A + (j ^ s);
 }
 
-template <int N, int CL>
-__global__ void __launch_bounds__(YZ<N, CL>::NT, 2) k_yzpass(Fields fp0, int region) {
-  using Y = YZ<N, CL>;
-  constexpr int M = Y::M, ZP = Y::ZP, H = Y::H, NT = Y::NT, FC = Y::FC, LP = Y::LP;
-  constexpr int R1 = Y::R1, R2 = Y::R2, MR1 = Y::MR1, MR2 = Y::MR2;
+template <int N, int NW>
+__global__ void __launch_bounds__(YZ<N, NW>::NT, YZ<N, NW>::MIN_BLOCKS) k_yzpass(Fields fp0, int region) {
+  using Y = YZ<N, NW>;
+  constexpr int A = Y::A, B = Y::B, ZP = Y::ZP, SP = Y::SP, H = Y::H, NT = Y::NT, COLS = Y::COLS;
   const Fields fp = at_chain(fp0, blockIdx.y);
   extern __shared__ __align__(128) unsigned char smem[];
   float2* blk = reinterpret_cast<float2*>(smem);
-  float2* ex = reinterpret_cast<float2*>(smem + Y::OFF_EX);
-  float2* twN = reinterpret_cast<float2*>(smem + Y::OFF_TWN);
-  float2* twM = reinterpret_cast<float2*>(smem + Y::OFF_TWM);
-  double* red = reinterpret_cast<double*>(smem + Y::OFF_RED);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + Y::OFF_BAR);
-  int* s_lo = reinterpret_cast<int*>(smem + Y::OFF_SPAN);
-  int* s_hi = s_lo + M;
-  const int t = threadIdx.x;
-  const int r = CL > 1 ? (int)(blockIdx.x % CL) : 0;     // rank in the cluster (cluster along x)
-  const int plane = (int)blockIdx.x / CL;
-  DevState* ds = fp.ds;
-  if (ds->jreuse) return;         // force stage reused by the jump (uniform)
+  float2* tw = reinterpret_cast<float2*>(smem + Y::OFF_TW);
+  float2* twa = reinterpret_cast<float2*>(smem + Y::OFF_TA);
+  float2* twb = reinterpret_cast<float2*>(smem + Y::OFF_TB);
+  __shared__ int s_lo[N], s_hi[N];
+  __shared__ float s_red[2 * Y::NW];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int plane = (int)blockIdx.x;
   float2* Wp = fp.W + (long long)plane * N * ZP;
+  // the first task's loads of the inverse y transform go out before anything waits
+  // (a plane without support, which does not need them, is rare)
+  float2 v0[B];
+  if (t < Y::T1) {
+#pragma unroll
+    for (int b = 0; b < B; ++b) v0[b] = Wp[(t / COLS + A * b) * ZP + t % COLS];
+  }
+  if (fp.ds->jreuse) return;      // force stage reused by the jump (uniform)
 
-  // ---- supports [lo, hi) of a and c on the z lines of this CTA (local row i is
-  // y = CL i + r); outside them g = 0
+  // ---- supports [lo, hi) of a and c on the z lines; outside them g = 0
   bool mine = false;
   const int2* span = survey(fp).span;
-  for (int i = t; i < M; i += NT) {
+  for (int i = t; i < N; i += NT) {
     int lo = 0, hi = N;
     if (span) {
-      const int2 sp = span[(long long)plane * N + CL * i + r];
+      const int2 sp = span[(long long)plane * N + i];
       lo = N - sp.x;
       hi = sp.y;
     }
@@ -107,256 +98,243 @@ __global__ void __launch_bounds__(YZ<N, CL>::NT, 2) k_yzpass(Fields fp0, int reg
     s_hi[i] = hi;
     mine |= hi > lo;
   }
-  if (t == 0) {
-    mbar_init(bar, 1);
-    mbar_fence_init();
+  for (int i = t; i < N; i += NT) {
+    tw[i] = fp.tw[i];
+    twa[i] = fp.tw[(i / A) * (i % A)];
+    twb[i] = fp.tw[(i / B) * (i % B)];
   }
-  const bool any_support = __syncthreads_or(mine);
-  if constexpr (CL == 1) {
+  if (!__syncthreads_or(mine)) {
     // a plane without support has g = 0 on every line: a zero force, W not read
-    if (!any_support) {
-      for (int e = t; e < Y::E; e += NT)
-        if (e % ZP <= H) Wp[e] = make_float2(0.f, 0.f);
-      if (region >= 0 && t == 0) fp.part[region + blockIdx.x] = 0.0;
-      return;
+    for (int e = t; e < N * ZP; e += NT)
+      if (e % ZP <= H) Wp[e] = make_float2(0.f, 0.f);
+    if (region >= 0 && t == 0) fp.part[region + plane] = 0.0;
+    return;
+  }
+
+  // ---- inverse y transform, first half: rows j + A b of W -> t[j][c] in row j + A c
+  for (int q = t; q < Y::T1; q += NT) {
+    const int j = q / COLS, col = q - j * COLS;
+    if (q != t) {
+#pragma unroll
+      for (int b = 0; b < B; ++b) v0[b] = Wp[(j + A * b) * ZP + col];
+    }
+    Dft<B, INV>::run(v0);
+    blk[j * SP + col] = v0[0];
+#pragma unroll
+    for (int c = 1; c < B; ++c) {
+      float2 w = tw[j * c];
+      w.y = -w.y;
+      blk[(j + A * c) * SP + col] = cmul(v0[c], w);
     }
   }
-
-  // ---- own rows ky in [r M, (r + 1) M): one bulk copy
-  if (t == 0) {
-    mbar_expect_tx(bar, (uint32_t)Y::BLK);
-    bulk_load(blk, Wp + (long long)r * M * ZP, (uint32_t)Y::BLK, bar);
+  __syncthreads();
+  // second half: y = c + B d into row d + A c
+  for (int q = t; q < Y::T2; q += NT) {
+    const int c = q / COLS, col = q - c * COLS;
+    float2* p = blk + A * c * SP + col;
+    float2 v[A];
+#pragma unroll
+    for (int j = 0; j < A; ++j) v[j] = p[j * SP];
+    Dft<A, INV>::run(v);
+#pragma unroll
+    for (int d = 0; d < A; ++d) p[d * SP] = v[d];
   }
-  for (int i = t; i < N; i += NT) twN[i] = fp.tw[i];
-  for (int i = t; i < M; i += NT) twM[i] = fp.tw[i * CL];
-  bool ok = mbar_wait(bar, 0);
-  ok = __syncthreads_and(ok);
-  if (!ok && t == 0) atomicOr(&ds->status, ST_TIMEOUT);
-  // no early return below: every CTA of the cluster must reach every cluster barrier
+  __syncthreads();
 
-  // ---- radix-CL combination of the cluster's row blocks (inverse sign)
-  if constexpr (CL > 1) {
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();                                      // every block has landed
-    const float2* peer[CL];
+  // ---- z lines [y0, y0 + 8) of this warp; pair i is (y0 + i, y0 + i + 4)
+  TwoSumAcc en;
+  const bool want_e = region >= 0;
+  for (int u = warp; u < Y::UNITS; u += NW) {
+    const int y0 = u * Y::LINES;
+    auto row = [&](int y) { return blk + (y / B + A * (y % B)) * SP; };
+    bool some = false;
+    if (lane < Y::LINES) some = s_hi[y0 + lane] > s_lo[y0 + lane];
+    if (!__any_sync(0xffffffffu, some)) {
+      for (int l = 0; l < Y::LINES; ++l) {
+        float2* r = row(y0 + l);
+        for (int k = lane; k <= H; k += 32) r[k] = make_float2(0.f, 0.f);
+      }
+    } else {
+      const int f1 = lane / A, a1 = lane % A;            // first inverse half and second forward half
+      const bool act1 = f1 < Y::PAIRS;
+      float2* ra = row(y0 + (act1 ? f1 : 0));
+      float2* rb = row(y0 + (act1 ? f1 : 0) + Y::PAIRS);
+      auto slot = [&](float2* pa, float2* pb, int pos) -> float2& { return pos < H ? pa[pos] : pb[pos - H]; };
+      {
+        float2 v[B];
+        if (act1) {
 #pragma unroll
-    for (int h = 0; h < CL; ++h) peer[h] = cluster.map_shared_rank(blk, h);
-#pragma unroll
-    for (int chunk = 0; chunk < 2; ++chunk) {
-      float2 acc[Y::CHUNK];
-#pragma unroll
-      for (int q = 0; q < Y::CHUNK; ++q) {
-        const int e = t + NT * (chunk * Y::CHUNK + q);
-        float2 s = make_float2(0.f, 0.f);
-        if (e < Y::E) {
-#pragma unroll
-          for (int h = 0; h < CL; ++h) s = cadd(s, root_cl<CL, INV>(peer[h][e], h * r));
-          float2 w = twN[(e / ZP) * r];
-          w.y = -w.y;                                    // e^{+2 pi i i r / N}
-          s = cmul(s, w);
+          for (int b = 0; b < B; ++b) {
+            const int k = a1 + A * b;
+            float2 xa, xb;
+            if (k <= H) {
+              xa = ra[k];
+              xb = rb[k];
+              if (k == 0 || k == H) { xa.y = 0.f; xb.y = 0.f; }
+            } else {
+              xa = cconj(ra[N - k]);
+              xb = cconj(rb[N - k]);
+            }
+            v[b] = make_float2(xa.x - xb.y, xa.y + xb.x);
+          }
+          Dft<B, INV>::run(v);
         }
-        acc[q] = s;
+        __syncwarp();
+        if (act1) {
+#pragma unroll
+          for (int c = 0; c < B; ++c) {
+            if (c) {
+              float2 w = twa[c * A + a1];
+              w.y = -w.y;
+              v[c] = cmul(v[c], w);
+            }
+            slot(ra, rb, zpos<N>(c, a1, f1)) = v[c];
+          }
+        }
       }
-      cluster.sync();                                    // all reads of this chunk are done
+      __syncwarp();
 #pragma unroll
-      for (int q = 0; q < Y::CHUNK; ++q) {
-        const int e = t + NT * (chunk * Y::CHUNK + q);
-        if (e < Y::E) blk[e] = acc[q];
+      for (int r = 0; r < Y::ZR; ++r) {
+        const int q = lane + 32 * r;
+        const int f = q / B, c = q - f * B;
+        const bool act = Y::ZT % 32 == 0 || q < Y::ZT;
+        const int ya = y0 + (act ? f : 0), yb = ya + Y::PAIRS;
+        float2* pa = row(ya);
+        float2* pb = row(yb);
+        float2 v[A];
+        if (act) {
+          const int loa = s_lo[ya], hia = s_hi[ya], lob = s_lo[yb], hib = s_hi[yb];
+          const long long la = ((long long)plane * N + ya) * N, lb = la + (long long)Y::PAIRS * N;
+          float aa[A], ca[A], ab[A], cb[A];
+#pragma unroll
+          for (int d = 0; d < A; ++d) {
+            const int n = c + B * d;
+            const bool ina = n >= loa && n < hia, inb = n >= lob && n < hib;
+            aa[d] = ina ? __ldg(fp.a + la + n) : 0.f;
+            ca[d] = ina ? __ldg(fp.c + la + n) : 0.f;
+            ab[d] = inb ? __ldg(fp.a + lb + n) : 0.f;
+            cb[d] = inb ? __ldg(fp.c + lb + n) : 0.f;
+          }
+#pragma unroll
+          for (int j = 0; j < A; ++j) v[j] = slot(pa, pb, zpos<N>(c, j, f));
+          Dft<A, INV>::run(v);
+          // here v[d] = y[c + B d]: real part line ya, imaginary part line yb
+#pragma unroll
+          for (int d = 0; d < A; ++d) {
+            const float da = v[d].x * fp.inv_nv, db = v[d].y * fp.inv_nv;
+            const float ga = fmaf(aa[d], da, -ca[d]), gb = fmaf(ab[d], db, -cb[d]);
+            if (want_e) {                               // a d^2 - 2 c d
+              en.add(da * (ga - ca[d]));
+              en.add(db * (gb - cb[d]));
+            }
+            v[d] = make_float2(ga, gb);
+          }
+          Dft<A, FWD>::run(v);
+        }
+        __syncwarp();
+        if (act) {
+#pragma unroll
+          for (int e = 0; e < A; ++e) slot(pa, pb, zpos<N>(c, e, f)) = e ? cmul(v[e], twb[e * B + c]) : v[e];
+        }
       }
-    }
-    __syncthreads();
-  }
-
-  // ---- inverse y transform of length M on every column of the block
-  for (int g = 0; g < Y::GROUPS; ++g) {
-    const int col = g * FC + t % FC, j = t / FC;
-    const bool cv = col < ZP;
-    float2 v[Y::MRMAX];
-    if (j < MR2) {
+      __syncwarp();
+      {
+        // second forward half, then the split into the two half spectra:
+        // G_a[k] = (Y[k] + conj Y[N-k]) / 2, G_b[k] = -i (Y[k] - conj Y[N-k]) / 2; Y[N - k]
+        // of k = e + A d sits in the pair's lane A - e as element B - 1 - d (or in the
+        // own element (B - d) mod B for e = 0)
+        float2 v[B];
+        if (act1) {
 #pragma unroll
-      for (int d = 0; d < MR1; ++d) v[d] = cv ? blk[(j + MR2 * d) * ZP + col] : make_float2(0.f, 0.f);
-    }
-    fft2<M, MR2, MR1, INV, MAP_COL, FC>(v, ex, twM, t);
-    if (j < MR1 && cv) {
+          for (int c = 0; c < B; ++c) v[c] = slot(ra, rb, zpos<N>(c, a1, f1));
+          Dft<B, FWD>::run(v);
+        }
+        __syncwarp();
+        const int src = act1 ? lane - a1 + (A - a1) % A : lane;
 #pragma unroll
-      for (int b = 0; b < MR2; ++b) blk[(j + MR1 * b) * ZP + col] = v[b];
+        for (int d = 0; d <= B / 2; ++d) {
+          const float2 snd = v[B - 1 - d];
+          float2 rcv;
+          rcv.x = __shfl_sync(0xffffffffu, snd.x, src);
+          rcv.y = __shfl_sync(0xffffffffu, snd.y, src);
+          const int k = a1 + A * d;
+          if (act1 && k <= H) {
+            const float2 yk = v[d];
+            const float2 ym = cconj(a1 == 0 ? v[(B - d) % B] : rcv);
+            ra[k] = make_float2(0.5f * (yk.x + ym.x), 0.5f * (yk.y + ym.y));
+            rb[k] = make_float2(0.5f * (yk.y - ym.y), -0.5f * (yk.x - ym.x));
+          }
+        }
+      }
     }
   }
   __syncthreads();
 
-  // ---- z lines: local row i is y = CL i + r.  C2R (two lines per complex
-  // transform), g = a delta - c and (1/2) sum (a delta^2 - 2 c delta), R2C.
-  double eacc = 0.0;
-  for (int q = 0; q < Y::ROUNDS; ++q) {
-    const int i0 = q * 2 * LP;
-    bool round_support = false;
+  // ---- forward y transform, first half: rows d + A c (y = c + B d) -> t[c][e] in row e + A c
+  for (int q = t; q < Y::T2; q += NT) {
+    const int c = q / COLS, col = q - c * COLS;
+    float2* p = blk + A * c * SP + col;
+    float2 v[A];
 #pragma unroll
-    for (int l = 0; l < 2 * LP; ++l) round_support |= s_hi[i0 + l] > s_lo[i0 + l];
-    if (!round_support) {
-      // every line of the round has g = 0: zero rows, no transforms
-      for (int i = t; i < 2 * LP * (H + 1); i += NT) {
-        const int l = i / (H + 1), k = i - l * (H + 1);
-        blk[(i0 + l) * ZP + k] = make_float2(0.f, 0.f);
-      }
-      __syncthreads();
-      continue;
-    }
-    float2 v[Y::RMAX];
-    {
-      const int f = t / R2, a = t % R2;
-      if (f < LP) {
-        const float2* ra = blk + (i0 + 2 * f) * ZP;
-        const float2* rb = ra + ZP;
+    for (int d = 0; d < A; ++d) v[d] = p[d * SP];
+    Dft<A, FWD>::run(v);
+    p[0] = v[0];
 #pragma unroll
-        for (int b = 0; b < R1; ++b) {
-          const int k = a + R2 * b;
-          float2 xa, xb;
-          if (k <= H) {
-            xa = ra[k];
-            xb = rb[k];
-            if (k == 0 || k == H) { xa.y = 0.f; xb.y = 0.f; }
-          } else {
-            xa = cconj(ra[N - k]);
-            xb = cconj(rb[N - k]);
-          }
-          v[b] = make_float2(xa.x - xb.y, xa.y + xb.x);
-        }
-      }
-    }
-    fft2<N, R2, R1, INV, MAP_ROW, LP>(v, ex, twN, t);
-    TwoSumAcc e;   // compensated: see TwoSumAcc
-    {
-      const int f = t / R1, c = t % R1;
-      if (f < LP) {
-        const long long la = ((long long)plane * N + (long long)CL * (i0 + 2 * f) + r) * N;
-        const long long lb = la + (long long)CL * N;
-        const float* pa = fp.a;
-        const float* pc = fp.c;
-        const int loa = s_lo[i0 + 2 * f], hia = s_hi[i0 + 2 * f];
-        const int lob = s_lo[i0 + 2 * f + 1], hib = s_hi[i0 + 2 * f + 1];
-#pragma unroll
-        for (int d = 0; d < R2; ++d) {
-          const int n = c + R1 * d;
-          const bool ina = n >= loa && n < hia, inb = n >= lob && n < hib;
-          const float aa = ina ? pa[la + n] : 0.f, ca = ina ? pc[la + n] : 0.f;
-          const float ab = inb ? pa[lb + n] : 0.f, cb = inb ? pc[lb + n] : 0.f;
-          const float da = v[d].x * fp.inv_nv, db = v[d].y * fp.inv_nv;
-          const float ga = fmaf(aa, da, -ca), gb = fmaf(ab, db, -cb);
-          if (region >= 0) {                             // a d^2 - 2 c d
-            e.add(da * (ga - ca));
-            e.add(db * (gb - cb));
-          }
-          v[d] = make_float2(ga, gb);
-        }
-      }
-    }
-    eacc += e.value();
-    fft2<N, R1, R2, FWD, MAP_ROW, LP>(v, ex, twN, t);
-    {
-      const int f = t / R2, c = t % R2;
-      if (f < LP) {
-#pragma unroll
-        for (int d = 0; d < R1; ++d) ex[f * N + c + R2 * d] = v[d];
-      }
-    }
-    __syncthreads();
-    for (int i = t; i < 2 * LP * (H + 1); i += NT) {
-      const int l = i / (H + 1), k = i - l * (H + 1);
-      const int f = l >> 1;
-      const float2 yk = ex[f * N + k];
-      const float2 ym = cconj(ex[f * N + (k == 0 ? 0 : N - k)]);
-      float2 g;
-      if ((l & 1) == 0) g = make_float2(0.5f * (yk.x + ym.x), 0.5f * (yk.y + ym.y));
-      else g = make_float2(0.5f * (yk.y - ym.y), -0.5f * (yk.x - ym.x));
-      blk[(i0 + l) * ZP + k] = g;
-    }
-    __syncthreads();
-  }
-  if (region >= 0) {
-    const double s = block_sum<NT>(0.5 * eacc, red);
-    if (t == 0) fp.part[region + blockIdx.x] = s;
-  }
-
-  // ---- forward y transform of length M on every column of the block
-  for (int g = 0; g < Y::GROUPS; ++g) {
-    const int col = g * FC + t % FC, j = t / FC;
-    const bool cv = col < ZP;
-    float2 v[Y::MRMAX];
-    if (j < MR1) {
-#pragma unroll
-      for (int b = 0; b < MR2; ++b) v[b] = cv ? blk[(j + MR1 * b) * ZP + col] : make_float2(0.f, 0.f);
-    }
-    fft2<M, MR1, MR2, FWD, MAP_COL, FC>(v, ex, twM, t);
-    if (j < MR2 && cv) {
-#pragma unroll
-      for (int d = 0; d < MR1; ++d) blk[(j + MR2 * d) * ZP + col] = v[d];
-    }
+    for (int e = 1; e < A; ++e) p[e * SP] = cmul(v[e], tw[c * e]);
   }
   __syncthreads();
-
-  // ---- radix-CL combination (forward sign) into rows ky = i + M r of W
-  if constexpr (CL > 1) {
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();                                      // every F_r' is complete
-    const float2* peer[CL];
+  // second half: ky = e + A f straight to W
+  for (int q = t; q < Y::T1; q += NT) {
+    const int e = q / COLS, col = q - e * COLS;
+    float2 v[B];
 #pragma unroll
-    for (int h = 0; h < CL; ++h) peer[h] = cluster.map_shared_rank(blk, h);
-    float2* out = Wp + (long long)r * M * ZP;
-    for (int e = t; e < Y::E; e += NT) {
-      const int i = e / ZP, kz = e - i * ZP;
-      if (kz > H) continue;
-      float2 s = make_float2(0.f, 0.f);
+    for (int c = 0; c < B; ++c) v[c] = blk[(e + A * c) * SP + col];
+    Dft<B, FWD>::run(v);
 #pragma unroll
-      for (int h = 0; h < CL; ++h) s = cadd(s, root_cl<CL, FWD>(cmul(peer[h][e], twN[i * h]), r * h));
-      out[e] = s;
-    }
-    cluster.sync();                                      // peers are done reading this block
-  } else {
-    for (int e = t; e < Y::E; e += NT) {
-      const int kz = e % ZP;
-      if (kz <= H) Wp[e] = blk[e];
-    }
+    for (int f = 0; f < B; ++f) Wp[(e + A * f) * ZP + col] = v[f];
+  }
+  if (want_e) {
+    TwoSumAcc h;                  // halving is exact
+    h.s = 0.5f * en.s;
+    h.c = 0.5f * en.c;
+    const double s = block_sum2<NT>(h, s_red);
+    if (t == 0) fp.part[region + plane] = s;
   }
 }
 
-template <int N, int CL>
+template <int N, int NW>
 void launch_yz(const Fields& f, int region, int nch, cudaStream_t s) {
-  using Y = YZ<N, CL>;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(N * CL, nch);
-  cfg.blockDim = dim3(Y::NT);
-  cfg.dynamicSmemBytes = Y::BYTES;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CL;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = CL > 1 ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, k_yzpass<N, CL>, f, region);
+  k_yzpass<N, NW><<<dim3(N, nch), YZ<N, NW>::NT, YZ<N, NW>::BYTES, s>>>(f, region);
 }
 
-template <int N, int CL>
+template <int N, int NW>
 bool set_yz(YzEntry* out) {
-  if (cudaFuncSetAttribute(k_yzpass<N, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)YZ<N, CL>::BYTES) !=
+  if (cudaFuncSetAttribute(k_yzpass<N, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)YZ<N, NW>::BYTES) !=
       cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  out->run = launch_yz<N, CL>;
-  out->tiles = N * CL;
+  out->run = launch_yz<N, NW>;
+  out->tiles = N;
   return true;
 }
 
 }  // namespace
 
-bool yz_table(int N, YzEntry* out) {
+// Two block widths.  With no more planes than SMs each SM holds one block, and a
+// block wide enough for one round of first-half y tasks (at 32^3: second-half) is
+// fastest.  With more planes narrower blocks, several to an SM, waste fewer lanes
+// in their last rounds and wait less at barriers: a Gibbs iteration of 32 chains
+// each of 32^3, 64^3 and 96^3 takes 8.83 ms with the wide blocks everywhere, 8.63 ms
+// with the narrow ones; of 24 chains of 128^3 9.09 ms with three narrow blocks per
+// SM (which spill) and 8.76 ms with two.
+bool yz_table(int N, int nch, int n_sm, YzEntry* out) {
+  const bool few = N * nch <= n_sm;
   switch (N) {
-    case 32: return set_yz<32, 1>(out);
-    case 64: return set_yz<64, 1>(out);
-    case 96: return set_yz<96, 1>(out);
-    case 128: return set_yz<128, 1>(out);
+    case 32: return few ? set_yz<32, 5>(out) : set_yz<32, 3>(out);
+    case 64: return few ? set_yz<64, 9>(out) : set_yz<64, 5>(out);
+    case 96: return few ? set_yz<96, 13>(out) : set_yz<96, 7>(out);
+    case 128: return few ? set_yz<128, 17>(out) : set_yz<128, 9>(out);
     default: return false;
   }
 }
