@@ -410,15 +410,13 @@ void prof_mark(bps_ctx* ctx, int k) {
 // ------------------------------------------------------------------ stages (all chains of a group)
 bps_status rebuild_chain(bps_ctx* ctx, int ch) {
   launch_rebuild(fields_at(ctx, ch), ctx->nv, region_offset(ctx, RG_RB), ctx->rebuild_blocks, 1, ctx->stream);
-  launch_abar(scalars_at(ctx, ch), region_offset(ctx, RG_RB), ctx->rebuild_blocks, 1, ctx->stream);
-  LAUNCHED(ctx, 2);
+  LAUNCHED(ctx, 1);
   return BPS_OK;
 }
 
 bps_status rebuild_all(bps_ctx* ctx) {
   launch_rebuild(fields(ctx), ctx->nv, region_offset(ctx, RG_RB), ctx->rebuild_blocks, ctx->batch, ctx->stream);
-  launch_abar(scalars(ctx), region_offset(ctx, RG_RB), ctx->rebuild_blocks, ctx->batch, ctx->stream);
-  LAUNCHED(ctx, 2);
+  LAUNCHED(ctx, 1);
   return BPS_OK;
 }
 
@@ -477,7 +475,7 @@ bps_status hmc_move(bps_ctx* ctx, bool advance) {
   P.x_final(f, region_offset(ctx, RG_FINAL), B, s);
   launch_move_end(sa, region_offset(ctx, RG_INIT), region_offset(ctx, RG_LIK0), region_offset(ctx, RG_FINAL),
                   region_offset(ctx, RG_LIK1), P.x_tiles, lik_tiles(ctx), B, s);
-  int n = 7 + L + (ctx->mnet ? 1 : 0);   // launch_move_end is two kernels
+  int n = 6 + L + (ctx->mnet ? 1 : 0);
   if (advance) {
     launch_advance(ctx->ds, B, s);
     ++n;
@@ -486,12 +484,13 @@ bps_status hmc_move(bps_ctx* ctx, bool advance) {
   return BPS_OK;
 }
 
-bps_status power_stage(bps_ctx* ctx, bool draw, bool advance) {
+// jump: 1 also starts the jump's HMC, 2 the same right after an HMC move (launch_power)
+bps_status power_stage(bps_ctx* ctx, bool draw, bool advance, int jump = 0) {
   Fields f = fields(ctx);
   ScalarArgs sa = scalars(ctx);
   const int B = ctx->batch;
   ctx->pt.x_binpow(f, region_offset(ctx, RG_BIN), B, ctx->stream);
-  launch_power(sa, region_offset(ctx, RG_BIN), ctx->pt.x_tiles, draw ? 1 : 0, B, ctx->stream);
+  launch_power(sa, region_offset(ctx, RG_BIN), ctx->pt.x_tiles, draw ? 1 : 0, jump, B, ctx->stream);
   int n = 2;
   if (advance) {
     launch_advance(ctx->ds, B, ctx->stream);
@@ -542,20 +541,15 @@ bps_status jump_gradient(bps_ctx* ctx, int kind) {
   return BPS_OK;
 }
 
-// sigma_current: DevState::sigma already holds the k-bin power of the current
-// field (the power draw of the same Gibbs iteration computed it, and the field
-// has not moved since), so the jump's mass needs no second reduction.
-bps_status jump_stage(bps_ctx* ctx, bool advance, bool sigma_current = false) {
-  ScalarArgs sa = scalars(ctx);
+// started: the power stage of the same Gibbs iteration has reduced sigma and
+// started the jump (the field has not moved since); W and the likelihood partials
+// of the move's last force evaluation are still in place.
+bps_status jump_stage(bps_ctx* ctx, bool advance, bool started = false) {
   cudaStream_t s = ctx->stream;
   const int B = ctx->batch;
   bps_status st = BPS_OK;
-  if (!sigma_current) st = power_stage(ctx, false, false);   // sigma of the current field (mass of the jump)
+  if (!started) st = power_stage(ctx, false, false, 1);   // sigma of the current field (mass of the jump)
   if (st != BPS_OK) return st;
-  // inside the Gibbs scan the jump follows the HMC move and the power draw, which
-  // leave W and the likelihood partials of the move's last force evaluation
-  launch_jump_begin(sa, sigma_current ? 1 : 0, B, s);
-  LAUNCHED(ctx, 1);
   const int L = ctx->cfg.jump_leapfrog;
   st = jump_gradient(ctx, J_FIRST);
   if (st != BPS_OK) return st;
@@ -577,7 +571,7 @@ bps_status jump_stage(bps_ctx* ctx, bool advance, bool sigma_current = false) {
 // sample into `rec` (slot DevState::rec_idx, layout [slot][chain][rec_len]).
 bps_status gibbs_once(bps_ctx* ctx, double* rec, int rec_len, long long iter_stride, bool jump) {
   bps_status st = hmc_move(ctx, false);
-  if (st == BPS_OK) st = power_stage(ctx, true, false);
+  if (st == BPS_OK) st = power_stage(ctx, true, false, jump ? 2 : 0);
   if (st == BPS_OK && jump) st = jump_stage(ctx, false, true);
   if (st == BPS_OK) st = bias_stage(ctx, false);
   if (st != BPS_OK) return st;
@@ -590,8 +584,7 @@ bps_status gibbs_once(bps_ctx* ctx, double* rec, int rec_len, long long iter_str
   }
   launch_record(scalars(ctx), rec, rec_len, iter_stride, ctx->chain_id.empty() ? 0 : ctx->chain_id[0], ctx->batch,
                 ctx->stream);
-  launch_advance(ctx->ds, ctx->batch, ctx->stream);
-  LAUNCHED(ctx, 2);
+  LAUNCHED(ctx, 1);
   return BPS_OK;
 }
 
@@ -1505,7 +1498,7 @@ bps_status window_power(bps_ctx* ctx, double* out, int out_stride, const std::ve
     ctx->pt.y_fwd(f, BUF_W, 1, s);
     ctx->pt.x_fwd(f, BUF_W, f.W, 1, s);
     ctx->pt.x_wpow(f, region_offset(ctx, RG_BIN), 1, s);
-    launch_power(scalars_at(ctx, ch), region_offset(ctx, RG_BIN), ctx->pt.x_tiles, 0, 1, s);
+    launch_power(scalars_at(ctx, ch), region_offset(ctx, RG_BIN), ctx->pt.x_tiles, 0, 0, 1, s);
     LAUNCHED(ctx, 5);
     std::vector<double> sig(MAXB);
     double abar = 0.0;

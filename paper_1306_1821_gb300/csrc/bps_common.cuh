@@ -250,17 +250,21 @@ struct DevState {
   double sumR[MAXS], sumB[MAXS], nobs[MAXS];
   double abar;                       // voxel mean of a = sum_l b_l^2 Nbar_l R^l
   // HMC move
-  double eps, u_acc, H0, H1, dH;
-  int accepted, cur, status, pad0;
+  double eps, log_u, H0, H1, dH;     // log_u: ln of the Metropolis uniform
+  int accepted, cur, status;
+  int mdone;                         // blocks of the running k_move_end that finished
   // jump move
-  double th[MAXB], rho[MAXB], mu[MAXB], jscale[MAXB], jgrad[MAXB];
-  double jeps, ju_acc, jH0, jH1, jdH, jlik;
+  double th[MAXB], th0[MAXB];        // ln P along the trajectory, and at its start
+  double rho[MAXB], inv_mu[MAXB];    // momenta and inverse masses
+  double je0[MAXB], je1[MAXB];       // kinetic and prior energy of each bin at the start and the end
+  double jeps, jlog_u, jH0, jH1, jdH, jlik0, jlik1;
   int jaccepted;
-  int jdone;                         // blocks of the running jump step that finished (k_jump_step)
+  int jdone;                         // blocks of the last jump step that finished (k_jump_step)
   // 1 while the jump's first gradient can reuse the force of the HMC move just
   // accepted (W and the likelihood partials of its last force evaluation are
   // those of the current field): its force stage is skipped
-  int jreuse, pad1;
+  int jreuse;
+  int rdone;                         // blocks of the running rebuild that finished (k_rebuild)
   // reductions handed between kernels
   double sigma[MAXB], sums[MAXS][3];
   double lik0, lik1;

@@ -30,31 +30,42 @@ __device__ double sum_partials(const double* p, int n, double* sh) {
 }
 
 // ------------------------------------------------------------------ HMC move
-__global__ void k_move_begin(ScalarArgs a0) {
+// The scalar kernels of a Gibbs iteration are chains of FP64 operations on a part
+// whose FP64 pipe is 1/64 of the FP32 one: a division or square root takes most
+// of a microsecond, a logarithm or exponential more.  So independent ones go to
+// different warps, variates that wait for nothing are drawn while the sums are
+// read, and small kernels that only consume what another one finishes are that
+// one's last block.
+
+// Per-bin tables of the move and its scalars: two warps per table column (a
+// division and a square root each), one for the step size and the Metropolis draw.
+__global__ void __launch_bounds__(288) k_move_begin(ScalarArgs a0) {
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   DevState* ds = a.ds;
-  const int t = threadIdx.x;
-  if (t == 0) {
-    P4 r = philox(0, ds->iteration, ST_HMC, 0, ds->seed);
-    ds->eps = a.eps_max * u52(r.w[0]);
-    ds->u_acc = u52(r.w[1]);
-  }
-  if (t < MAXB) {
-    if (t < a.n_bins) {
-      // lambda_m = P_m / V_cell (Eq. dens_prior in Fourier space); M = 1/lambda + abar (Eq. Mass_matrix)
-      const double il = ds->vc / ds->P[t];
-      const double M = il + ds->abar;
-      ds->inv_lambda[t] = (float)il;
-      ds->inv_M[t] = (float)(1.0 / M);
-      ds->sqrt_M[t] = (float)sqrt(M);
-    } else {
-      ds->inv_lambda[t] = 0.f;
-      ds->inv_M[t] = 0.f;
-      ds->sqrt_M[t] = 0.f;
+  const int t = threadIdx.x & 63, role = threadIdx.x >> 6;
+  if (role == 4) {
+    if (t == 0) {
+      P4 r = philox(0, ds->iteration, ST_HMC, 0, ds->seed);
+      ds->eps = a.eps_max * u52(r.w[0]);
+      ds->log_u = log(u52(r.w[1]));
     }
+    return;
+  }
+  if (role < 2) {
+    // lambda_m = P_m / V_cell (Eq. dens_prior in Fourier space); M = 1/lambda + abar (Eq. Mass_matrix)
+    const bool bin = t < a.n_bins;
+    const double il = bin ? ds->vc / ds->P[t] : 0.0;
+    const double M = il + ds->abar;
+    if (role == 0) {
+      ds->inv_lambda[t] = (float)il;
+      ds->inv_M[t] = bin ? (float)(1.0 / M) : 0.f;
+    } else {
+      ds->sqrt_M[t] = bin ? (float)sqrt(M) : 0.f;
+    }
+  } else {
     const double sc = t < a.n_mass ? ds->mass_scale[t] : 1.0;
-    ds->inv_ms[t] = (float)(1.0 / sc);
-    ds->sqrt_ms[t] = (float)sqrt(sc);
+    if (role == 2) ds->inv_ms[t] = (float)(1.0 / sc);
+    else ds->sqrt_ms[t] = (float)sqrt(sc);
   }
 }
 
@@ -62,10 +73,12 @@ __global__ void k_move_begin(ScalarArgs a0) {
 // The eight sums of a move, one block each (on different SMs: each sum is a
 // chain of FP64 additions), into the chain state's scratch: K0, E0, L0, K1, E1,
 // L1, G0, G1 (the kinetic, prior and likelihood energies at the start and the
-// end, and the two force norms of the leapfrog energy identity).
-__global__ void k_move_sums(ScalarArgs a0, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz) {
+// end, and the two force norms of the leapfrog energy identity).  The last block
+// to finish takes the Metropolis decision.
+__global__ void k_move_end(ScalarArgs a0, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz) {
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   __shared__ double sh[32];
+  DevState* ds = a.ds;
   const double h = 0.5 * a.inv_nv;
   const double* p = nullptr;
   int n = nx;
@@ -81,16 +94,15 @@ __global__ void k_move_sums(ScalarArgs a0, int r_init, int r_lik0, int r_final, 
     default: p = a.part + r_final + 2 * a.stride; scale = a.inv_nv; break;
   }
   const double s = sum_partials(p, n, sh);
-  if (threadIdx.x == 0) a.ds->scratch[blockIdx.x] = s * scale;
-}
-
-__global__ void k_move_end(ScalarArgs a0) {
-  const ScalarArgs a = chain_args(a0, blockIdx.y);
-  DevState* ds = a.ds;
   if (threadIdx.x == 0) {
-    const double K0 = ds->scratch[0], E0 = ds->scratch[1], L0 = ds->scratch[2];
-    const double K1 = ds->scratch[3], E1 = ds->scratch[4], L1 = ds->scratch[5];
-    const double G0 = ds->scratch[6], G1 = ds->scratch[7];
+    ds->scratch[blockIdx.x] = s * scale;
+    __threadfence();
+    if (atomicAdd(&ds->mdone, 1) != (int)gridDim.x - 1) return;
+    __threadfence();
+    ds->mdone = 0;
+    const double K0 = __ldcg(ds->scratch + 0), E0 = __ldcg(ds->scratch + 1), L0 = __ldcg(ds->scratch + 2);
+    const double K1 = __ldcg(ds->scratch + 3), E1 = __ldcg(ds->scratch + 4), L1 = __ldcg(ds->scratch + 5);
+    const double G0 = __ldcg(ds->scratch + 6), G1 = __ldcg(ds->scratch + 7);
     const double H0 = K0 + E0 + L0, H1 = K1 + E1 + L1;
     // H(end) - H(start) of Eq. acceptance_rule.  The potential of the density
     // move (Eq. Wiener_Posterior_psi with fixed P, b, Nbar) is exactly quadratic
@@ -114,7 +126,7 @@ __global__ void k_move_end(ScalarArgs a0) {
     if (!isfinite(dH) || !isfinite(H0) || !isfinite(H1)) {
       ds->status |= ST_NONFINITE;
     } else {
-      acc = log(ds->u_acc) < -dH;   // Eq. acceptance_rule, FP64
+      acc = ds->log_u < -dH;        // Eq. acceptance_rule, FP64
     }
     ds->accepted = acc;
     if (acc) {
@@ -129,22 +141,31 @@ __global__ void k_move_end(ScalarArgs a0) {
 // Gamma(shape) by Marsaglia & Tsang (ACM TOMS 2000); attempt j of bin m reads
 // Philox block (m, iteration, ST_POWER, j): words 0,1 -> normal, word 2 -> uniform;
 // shape < 1 uses Gamma(shape + 1) U^(1/shape) with U from word 3 of attempt 0.
+// Called by all 32 lanes of one warp (identical arguments): lane q makes the
+// attempts q and 32 + q, the first accepted one counts; every lane returns it.
 __device__ double gamma_mt(double shape, uint64_t seed, uint64_t it, int m, int* fail) {
   const bool boost = shape < 1.0;
   const double aa = boost ? shape + 1.0 : shape;
   const double d = aa - 1.0 / 3.0;
   const double c = 1.0 / sqrt(9.0 * d);
+  const int lane = threadIdx.x & 31;
   double val = d;
   bool ok = false;
-  for (int j = 0; j < MAX_ATTEMPTS && !ok; ++j) {
-    P4 r = philox((uint64_t)m, it, ST_POWER, (uint64_t)j, seed);
+  for (int j0 = 0; j0 < MAX_ATTEMPTS && !ok; j0 += 32) {
+    P4 r = philox((uint64_t)m, it, ST_POWER, (uint64_t)(j0 + lane), seed);
     const double z = normal64(r.w[0], r.w[1]);
     const double t = 1.0 + c * z;
-    if (t <= 0.0) continue;
-    const double v = t * t * t;
-    const double u = u52(r.w[2]);
-    if (log(u) < 0.5 * z * z + d - d * v + d * log(v)) {
-      val = d * v;
+    bool acc = false;
+    double mine = 0.0;
+    if (t > 0.0) {
+      const double v = t * t * t;
+      const double u = u52(r.w[2]);
+      acc = log(u) < 0.5 * z * z + d - d * v + d * log(v);
+      mine = d * v;
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, acc);
+    if (who) {
+      val = __shfl_sync(0xffffffffu, mine, __ffs((int)who) - 1);
       ok = true;
     }
   }
@@ -157,22 +178,78 @@ __device__ double gamma_mt(double shape, uint64_t seed, uint64_t it, int m, int*
 }
 
 // block m: sigma_m = (V_cell/N^3) sum_{k in m} w |delta_k|^2; then (draw) P_m = sigma_m / x,
-// x ~ chi^2_beta = 2 Gamma(beta/2), beta = n_m + 2 alpha - 2 (Sec. 4.2, Eq. XI_SQUARE)
-__global__ void k_power(ScalarArgs a0, int region, int nx, int draw) {
+// x ~ chi^2_beta = 2 Gamma(beta/2), beta = n_m + 2 alpha - 2 (Sec. 4.2, Eq. XI_SQUARE); then
+// (jump) the start of the jump's HMC in theta = ln P with the whitened field fixed
+// (Sec. 4.3, App. C), whose mass mu_m = max(1, abar P_ref_m sigma_m / (4 V_cell P_m)) is
+// built from the whitened field and a fixed reference spectrum, never from the current P.
+// Eight warps sum; a ninth draws the Gamma variate and a tenth the jump's normal
+// meanwhile (neither depends on the sum).
+// jump = 2: the jump directly follows this iteration's HMC move, so after an accepted
+// move its first gradient can take the move's last force.
+__global__ void __launch_bounds__(320) k_power(ScalarArgs a0, int region, int nx, int draw, int jump) {
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   __shared__ double sh[32];
+  __shared__ double s_gamma, s_z, s_sigma, s_P;
+  __shared__ int s_fail;
   DevState* ds = a.ds;
-  const int m = blockIdx.x;
-  const double s = sum_partials(a.part + region + (size_t)m * a.stride, nx, sh);
-  if (threadIdx.x == 0) {
+  const int m = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  double v = 0.0;
+  if (warp < 8) {
+    const double* p = a.part + region + (size_t)m * a.stride;
+    for (int i = t; i < nx; i += 256) v += p[i];
+    v = warp_sum(v);
+    if (lane == 0) sh[warp] = v;
+  } else if (warp == 8) {
+    if (draw) {
+      int fail = 0;
+      const double g = gamma_mt(0.5 * (ds->nmodes[m] + 2.0 * a.alpha - 2.0), ds->seed, ds->iteration, m, &fail);
+      if (lane == 0) {
+        s_gamma = g;
+        s_fail = fail;
+      }
+    }
+  } else if (jump) {
+    const P4 r = philox((uint64_t)m, ds->iteration, ST_JUMP_MOM, 0, ds->seed);
+    const double z = normal64(r.w[0], r.w[1]);
+    if (lane == 0) s_z = z;
+  }
+  __syncthreads();
+  if (t == 0) {
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s += sh[i];
     const double sigma = s * ds->vc * a.inv_nv;
     ds->sigma[m] = sigma;
+    double P = ds->P[m];
     if (draw) {
-      const double beta = ds->nmodes[m] + 2.0 * a.alpha - 2.0;
-      int fail = 0;
-      const double g = gamma_mt(0.5 * beta, ds->seed, ds->iteration, m, &fail);
-      if (fail || !(sigma > 0.0)) atomicOr(&ds->status, ST_DRAW_FAIL);
-      else ds->P[m] = sigma / (2.0 * g);
+      if (s_fail || !(sigma > 0.0)) {
+        atomicOr(&ds->status, ST_DRAW_FAIL);
+      } else {
+        P = sigma / (2.0 * s_gamma);
+        ds->P[m] = P;
+      }
+    }
+    s_sigma = sigma;
+    s_P = P;
+  }
+  if (!jump) return;
+  __syncthreads();
+  if (lane == 0) {
+    if (warp == 0 || warp == 1) {
+      const double mu = fmax(1.0, ds->abar * ds->P_ref[m] * s_sigma / (4.0 * ds->vc * s_P));
+      if (warp == 0) ds->rho[m] = sqrt(mu) * s_z;
+      else ds->inv_mu[m] = 1.0 / mu;
+    } else if (warp == 2) {
+      const double th = log(s_P);
+      ds->th[m] = th;
+      ds->th0[m] = th;
+      ds->js[m] = 1.f;
+    } else if (warp == 3 && m == 0) {
+      ds->jreuse = jump == 2 && ds->accepted;
+      const P4 r = philox(0, ds->iteration, ST_JUMP, 0, ds->seed);
+      ds->jeps = a.jeps_max * u52(r.w[0]);
+      ds->jlog_u = log(u52(r.w[1]));
+      ds->jaccepted = 0;
     }
   }
 }
@@ -182,66 +259,64 @@ __global__ void k_power(ScalarArgs a0, int region, int nx, int draw) {
 // omega = sqrt(A B), y = x/eta (p >= 0) or eta/x (p < 0) has density
 // h(y) ~ y^(lam-1) exp(-omega (y + 1/y)/2), lam = |p|; sampled by the
 // ratio-of-uniforms method with mode shift (Kinderman & Monahan 1977), the
-// bounding rectangle found by bisection, everything in log space about the mode.
-__device__ double gig_logh(double y, double lam, double om, double m) {
-  return (lam - 1.0) * log1p((y - m) / m) - 0.5 * om * (y - m) * (1.0 - 1.0 / (y * m));
-}
-__device__ double gig_dphi(double y, double lam, double om, double m) {
-  return 1.0 / (y - m) + 0.5 * ((lam - 1.0) / y - 0.5 * om + 0.5 * om / (y * y));
-}
-
-// Root of gig_dphi in (lo, hi), found by the 32 lanes of a warp together:
-// each round evaluates 32 interior points, keeps the one gap where the sign
-// turns and shrinks the interval 33-fold (12 rounds reach FP64 resolution).
-// `neg_right`: the right-hand side of the root is where gig_dphi < 0 (else
-// where it is <= 0).  All lanes return the same value.
-__device__ double warp_root(double lo, double hi, bool neg_right, double lam, double om, double m) {
-  const int lane = threadIdx.x & 31;
-  for (int round = 0; round < 16; ++round) {
-    const double w = (hi - lo) / 33.0;
-    if (!(w > 0.0)) break;
-    const double x = lo + w * (double)(lane + 1);
-    const double d = gig_dphi(x, lam, om, m);
-    const unsigned right = __ballot_sync(0xffffffffu, neg_right ? (d < 0.0) : !(d > 0.0));
-    const int k = right ? __ffs(right) - 1 : 32;        // first point on the right-hand side
-    const double nlo = lo + w * (double)k;
-    const double nhi = k == 32 ? hi : lo + w * (double)(k + 1);
-    if (!(nlo > lo || nhi < hi)) break;
-    lo = nlo;
-    hi = nhi;
-  }
-  return 0.5 * (lo + hi);
+// bounding rectangle from the extremes of (y - m) sqrt(h(y)), everything in log
+// space about the mode m.  ln h(m + d) - ln h(m):
+__device__ double gig_logh(double d, double lam, double om, double m) {
+  return (lam - 1.0) * log1p(d / m) - 0.5 * om * d * (1.0 - 1.0 / ((m + d) * m));
 }
 
 // Called by all 32 lanes of one warp (identical arguments); every lane returns
-// the same draw.
-__device__ double gig_draw(double p, double A, double B, uint64_t seed, uint64_t it, int l, int* fail) {
+// the same draw.  lu, u, w: ln u, u and the second uniform of each of the 64
+// attempts (shared memory).
+//
+// The extremes: d/dy ln((y - m) sqrt(h)) = 0, with the mode's equation
+// (lam - 1) m = (omega / 2)(m^2 - 1), is (omega / 4)(y - m)^2 (y + 1/m) = y^2, or
+// G(d) = d -+ 2 y / sqrt(omega (y + 1/m)) = 0 with y = m + d, one root on either
+// side of the mode.  G rises through its root, nearly linearly for the peaked
+// densities of a survey: Newton's method within a bracket, the upper root in the
+// lower half of the warp and the lower root in the upper half.  (y - m) sqrt(h) is
+// stationary there, so a relative step of 1e-9 leaves it exact to FP64.  A search
+// by 32-point section took 12 to 16 rounds for each root, two thirds of the 66 to
+// 75 us of this kernel.
+__device__ double gig_draw(double p, double A, double B, const double* lu, const double* u, const double* w,
+                           int* fail) {
+  const int lane = threadIdx.x & 31;
   const double lam = fabs(p);
   const double om = sqrt(A * B);
   const double eta = sqrt(B / A);
   const double q = lam - 1.0;
   const double sq = sqrt(q * q + om * om);
   const double m = q >= 0.0 ? (q + sq) / om : om / (sq - q);
-  // upper extreme of (y - m) sqrt(h(y)/h(m))
-  double step = m, hi = m + step;
-  for (int i = 0; i < 200 && gig_dphi(hi, lam, om, m) > 0.0; ++i) {
-    step *= 2.0;
-    hi = m + step;
+  const double im = 1.0 / m;
+  const bool up = lane < 16;
+  double lo = up ? 0.0 : -m, hi = up ? 1.7e308 : 0.0;
+  double d = 2.0 * m * rsqrt(om * (m + im));
+  if (!up) d = d < m ? -d : -0.5 * m;
+  for (int i = 0; i < 200; ++i) {
+    const double y = m + d;
+    const double r = rsqrt(om * (y + im));
+    const double f = 2.0 * y * r;
+    const double G = up ? d - f : d + f;
+    const double df = 2.0 * r - y * om * r * r * r;
+    if (G < 0.0) lo = d;
+    else hi = d;
+    double nd = d - G / (up ? 1.0 - df : 1.0 + df);
+    if (!(nd > lo && nd < hi)) nd = up && hi > 1e308 ? 2.0 * d : 0.5 * (lo + hi);
+    const bool done = !(fabs(nd - d) > 1e-9 * fabs(d));
+    d = nd;
+    if (__all_sync(0xffffffffu, done)) break;
   }
-  const double yp = warp_root(m, hi, false, lam, om, m);
-  const double vp = (yp - m) * exp(0.5 * gig_logh(yp, lam, om, m));
-  const double ym = warp_root(0.0, m, true, lam, om, m);
-  const double vm = ym > 0.0 ? (ym - m) * exp(0.5 * gig_logh(ym, lam, om, m)) : -m;
+  const double ext = m + d > 0.0 ? d * exp(0.5 * gig_logh(d, lam, om, m)) : -m;
+  const double vp = __shfl_sync(0xffffffffu, ext, 0), vm = __shfl_sync(0xffffffffu, ext, 16);
   double y = m;
   bool ok = false;
-  for (int j = 0; j < MAX_ATTEMPTS && !ok; ++j) {
-    P4 r = philox((uint64_t)l, it, ST_NBAR, (uint64_t)j, seed);
-    const double u = u52(r.w[0]);
-    const double v = vm + (vp - vm) * u52(r.w[1]);
-    const double yy = v / u + m;
-    if (yy <= 0.0) continue;
-    if (2.0 * log(u) <= gig_logh(yy, lam, om, m)) {
-      y = yy;
+  for (int j0 = 0; j0 < MAX_ATTEMPTS && !ok; j0 += 32) {   // lane q makes the attempts q and 32 + q
+    const int j = j0 + lane;
+    const double dd = (vm + (vp - vm) * w[j]) / u[j];
+    const bool acc = dd + m > 0.0 && 2.0 * lu[j] <= gig_logh(dd, lam, om, m);
+    const unsigned who = __ballot_sync(0xffffffffu, acc);
+    if (who) {
+      y = m + __shfl_sync(0xffffffffu, dd, __ffs((int)who) - 1);
       ok = true;
     }
   }
@@ -251,66 +326,80 @@ __device__ double gig_draw(double p, double A, double B, uint64_t seed, uint64_t
 
 // block l: S1 = sum N delta, S2 = sum R delta, S3 = sum R delta^2; then
 // b_l ~ N(D/C, 1/C), C = Nbar S3, D = S1 - Nbar S2 (Sec. 3.5, App. B; skipped for
-// the fixed index) and Nbar_l ~ GIG(1 - N_obs/2, sum R + 2 b S2 + b^2 S3, sum N^2/R)
-__global__ void k_bias_nbar(ScalarArgs a0, int region, int nz) {
+// the fixed index) and Nbar_l ~ GIG(1 - N_obs/2, sum R + 2 b S2 + b^2 S3, sum N^2/R).
+// Eight warps sum the three quantities together; a ninth draws the bias normal and
+// two more the uniforms of the GIG attempts (attempt j reads Philox block (l,
+// iteration, ST_NBAR, j): word 0 gives u, word 1 the second uniform).
+// 66-75 us a launch with the section search and serial attempts, now 17-20 us.
+__global__ void __launch_bounds__(352) k_bias_nbar(ScalarArgs a0, int region, int nz) {
   const ScalarArgs a = chain_args(a0, blockIdx.y);
-  __shared__ double sh[32];
+  __shared__ double sh[3][8];
+  __shared__ double s_S[3], s_z, s_lu[MAX_ATTEMPTS], s_u[MAX_ATTEMPTS], s_w[MAX_ATTEMPTS];
   DevState* ds = a.ds;
-  const int l = blockIdx.x;
+  const int l = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   if (l >= ds->nsub) return;
-  double S[3];
-  for (int q = 0; q < 3; ++q) S[q] = sum_partials(a.part + region + (size_t)(3 * l + q) * a.stride, nz, sh);
-  // the sums are valid in thread 0: hand them to the first warp, which draws
-  // together (the GIG bounds are found lane-parallel); lane 0 writes
-  if (threadIdx.x == 0) {
-    sh[0] = S[0];
-    sh[1] = S[1];
-    sh[2] = S[2];
+  const uint64_t it = ds->iteration;
+  if (warp < 8) {
+    const double* p = a.part + region + (size_t)3 * l * a.stride;
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0;
+    for (int i = t; i < nz; i += 256) {
+      v0 += p[i];
+      v1 += p[a.stride + i];
+      v2 += p[2 * (size_t)a.stride + i];
+    }
+    v0 = warp_sum(v0);
+    v1 = warp_sum(v1);
+    v2 = warp_sum(v2);
+    if (lane == 0) {
+      sh[0][warp] = v0;
+      sh[1][warp] = v1;
+      sh[2][warp] = v2;
+    }
+  } else if (warp == 8) {
+    const P4 r = philox((uint64_t)l, it, ST_BIAS, 0, ds->seed);
+    const double z = normal64(r.w[0], r.w[1]);
+    if (lane == 0) s_z = z;
+  } else {
+    const int j = (warp - 9) * 32 + lane;
+    const P4 r = philox((uint64_t)l, it, ST_NBAR, (uint64_t)j, ds->seed);
+    const double u = u52(r.w[0]);
+    s_u[j] = u;
+    s_w[j] = u52(r.w[1]);
+    s_lu[j] = log(u);
   }
   __syncthreads();
-  if (threadIdx.x < 32) {
-    S[0] = sh[0];
-    S[1] = sh[1];
-    S[2] = sh[2];
-    const bool lead = threadIdx.x == 0;
-    const uint64_t it = ds->iteration;
-    if (lead) {
-      ds->sums[l][0] = S[0];
-      ds->sums[l][1] = S[1];
-      ds->sums[l][2] = S[2];
-    }
-    double b = ds->b[l];
-    const double nb = ds->nbar[l];
-    int fail = 0;
-    if (l != a.fixed_bias) {
-      const double C = nb * S[2];
-      const double D = S[0] - nb * S[1];
-      P4 r = philox((uint64_t)l, it, ST_BIAS, 0, ds->seed);
-      const double z = normal64(r.w[0], r.w[1]);
-      if (C > 0.0) b = D / C + z / sqrt(C);
-      else fail = 1;
-    }
-    const double A = ds->sumR[l] + 2.0 * b * S[1] + b * b * S[2];
-    const double p = 1.0 - 0.5 * ds->nobs[l];
-    double x = nb;
-    if (A > 0.0 && ds->sumB[l] > 0.0) x = gig_draw(p, A, ds->sumB[l], ds->seed, it, l, &fail);
+  if (warp != 0) return;
+  if (lane < 3) {
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s += sh[lane][i];
+    s_S[lane] = s;
+    ds->sums[l][lane] = s;
+  }
+  __syncwarp();
+  const double S0 = s_S[0], S1 = s_S[1], S2 = s_S[2];
+  double b = ds->b[l];
+  const double nb = ds->nbar[l];
+  int fail = 0;
+  if (l != a.fixed_bias) {
+    const double C = nb * S2;
+    const double D = S0 - nb * S1;
+    if (C > 0.0) b = D / C + s_z / sqrt(C);
     else fail = 1;
-    if (lead) {
-      if (fail || !isfinite(b) || !isfinite(x)) {
-        atomicOr(&ds->status, ST_DRAW_FAIL);
-      } else {
-        ds->b[l] = b;
-        ds->nbar[l] = x;
-      }
+  }
+  const double A = ds->sumR[l] + 2.0 * b * S1 + b * b * S2;
+  const double p = 1.0 - 0.5 * ds->nobs[l];
+  double x = nb;
+  if (A > 0.0 && ds->sumB[l] > 0.0) x = gig_draw(p, A, ds->sumB[l], s_lu, s_u, s_w, &fail);
+  else fail = 1;
+  if (lane == 0) {
+    if (fail || !isfinite(b) || !isfinite(x)) {
+      atomicOr(&ds->status, ST_DRAW_FAIL);
+    } else {
+      ds->b[l] = b;
+      ds->nbar[l] = x;
     }
   }
-}
-
-__global__ void k_abar(ScalarArgs a0, int region, int nblk) {
-  const ScalarArgs a = chain_args(a0, blockIdx.y);
-  __shared__ double sh[32];
-  const double s = sum_partials(a.part + region, nblk, sh);
-  if (threadIdx.x == 0) a.ds->abar = s * a.inv_nv;
 }
 
 // ------------------------------------------------------------------ survey commit
@@ -351,127 +440,92 @@ __global__ void k_commit_data(DevState* ds0, const double* part0, long long cstr
 }
 
 // ------------------------------------------------------------------ jump move
-// HMC in theta = ln P with the whitened field fixed (Sec. 4.3, App. C).
-// Mass mu_m = max(1, abar P_ref_m sigma_m / (4 V_cell P_m)): built from the
-// whitened field and a fixed reference spectrum, never from the current P.
-// reuse: the jump directly follows this iteration's HMC move and power draw, so
-// after an accepted move the first gradient can take the move's last force.
-__global__ void k_jump_begin(ScalarArgs a0, int reuse) {
-  const ScalarArgs a = chain_args(a0, blockIdx.y);
-  DevState* ds = a.ds;
-  const int m = threadIdx.x;
-  const uint64_t it = ds->iteration;
-  if (m == 0) {
-    ds->jreuse = reuse && ds->accepted;
-    P4 r = philox(0, it, ST_JUMP, 0, ds->seed);
-    ds->jeps = a.jeps_max * u52(r.w[0]);
-    ds->ju_acc = u52(r.w[1]);
-    ds->jaccepted = 0;
-  }
-  if (m < MAXB) {
-    if (m < a.n_bins) {
-      const double mu = fmax(1.0, ds->abar * ds->P_ref[m] * ds->sigma[m] / (4.0 * ds->vc * ds->P[m]));
-      P4 r = philox((uint64_t)m, it, ST_JUMP_MOM, 0, ds->seed);
-      ds->mu[m] = mu;
-      ds->rho[m] = sqrt(mu) * normal64(r.w[0], r.w[1]);
-      ds->th[m] = log(ds->P[m]);
-    }
-    ds->js[m] = 1.f;
-  }
-}
-
-// Leapfrog update of the jump's HMC in theta after a gradient evaluation (kind:
-// J_FIRST half kick and drift with the starting energy, J_MID kick and drift,
-// J_LAST half kick, final energy and Metropolis test).  Threads m < n_bins own
-// bin m; every thread of the block takes part in the barriers.
-__device__ void jump_update(const ScalarArgs& a, int kind, double* sh) {
-  DevState* ds = a.ds;
-  const int m = threadIdx.x;
-  const double eps = ds->jeps;
-  const bool act = m < a.n_bins;
-  double kin = 0.0, pri = 0.0;
-  double rho = act ? ds->rho[m] : 0.0, th = act ? ds->th[m] : 0.0;
-  // written by the other blocks of this launch: read past L1
-  const double mu = act ? ds->mu[m] : 1.0, g = act ? __ldcg(&ds->jgrad[m]) : 0.0;
-  if (kind == J_FIRST && act) {
-    kin = 0.5 * rho * rho / mu;
-    pri = (a.alpha - 1.0) * th;
-  }
-  if (act) {
-    const double ek = (kind == J_MID) ? eps : 0.5 * eps;
-    rho -= ek * g;
-    if (kind != J_LAST) th += eps * rho / mu;
-  }
-  if (kind == J_LAST && act) {
-    kin = 0.5 * rho * rho / mu;
-    pri = (a.alpha - 1.0) * th;
-  }
-  // 64-thread sums (two warps)
-  double e = kin + pri;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) e += __shfl_down_sync(0xffffffffu, e, o);
-  __syncthreads();
-  if ((m & 31) == 0) sh[m >> 5] = e;
-  __syncthreads();
-  const double E = sh[0] + sh[1];   // bins live in the first two warps (n_bins <= 64)
-  if (act) {
-    ds->rho[m] = rho;
-    ds->th[m] = th;
-    ds->js[m] = (float)sqrt(exp(th) / ds->P[m]);
-  }
-  const double jlik = __ldcg(&ds->jlik);
-  if (kind == J_FIRST && m == 0) ds->jH0 = E + jlik;
-  if (kind == J_LAST) {
-    __shared__ int s_acc;
-    if (m == 0) {
-      const double H1 = E + jlik;
-      const double dH = H1 - ds->jH0;
-      ds->jH1 = H1;
-      ds->jdH = dH;
-      int acc = 0;
-      if (!isfinite(dH)) ds->status |= ST_NONFINITE;
-      else acc = log(ds->ju_acc) < -dH;
-      ds->jaccepted = acc;
-      s_acc = acc;
-    }
-    __syncthreads();
-    if (act && s_acc) ds->P[m] = exp(th);
-  }
-}
-
-
-// One leapfrog step of the jump after its gradient evaluation, in one launch:
-// blocks m < n_bins reduce the gradient d psi_J / d theta_m = (alpha - 1) +
-// (1/2N^3) sum_{k in m} w Re(conj(g) delta), block n_bins (launched for J_FIRST
-// and J_LAST only, whose update needs the energy) the likelihood energy at
-// theta; the last block to finish (a counter in the chain state, which it
-// resets) then applies the update of `kind`.
-__global__ void k_jump_step(ScalarArgs a0, int r_grad, int nx, int r_lik, int r_lik_move, int nz, int kind) {
+// HMC in theta = ln P with the whitened field fixed (Sec. 4.3, App. C), started by k_power.
+//
+// One leapfrog step after its gradient evaluation.  Block m < n_bins reduces the
+// gradient d psi_J / d theta_m = (alpha - 1) + (1/2N^3) sum_{k in m} w Re(conj(g) delta)
+// and updates bin m, which needs no other bin: J_FIRST half kick and drift (keeping
+// the bin's starting energy), J_MID kick and drift, J_LAST half kick and final
+// energy.  Block n_bins (J_FIRST and J_LAST) reduces the likelihood energy at theta.
+// Only J_LAST joins the bins: its last block to finish sums the energies and takes
+// the Metropolis decision.  The field scale sqrt(exp(theta) / P) is
+// exp((theta - theta_0) / 2), one FP64 exponential instead of an exponential, a
+// division and a square root.  9.0 us a launch at 128^3 with every step joined in
+// its last block, now 5.9 us.
+__global__ void __launch_bounds__(256) k_jump_step(ScalarArgs a0, int r_grad, int nx, int r_lik, int r_lik_move, int nz,
+                                                   int kind) {
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   __shared__ double sh[32];
-  __shared__ int s_last;
+  __shared__ int s_last, s_acc;
   DevState* ds = a.ds;
-  const int m = blockIdx.x;
+  const int m = blockIdx.x, t = threadIdx.x;
   if (m < a.n_bins) {
+    double rho = 0.0, th = 0.0, im = 0.0, th0 = 0.0, eps = 0.0;
+    if (t == 0) {                 // in flight with the partial sums
+      rho = ds->rho[m];
+      th = ds->th[m];
+      im = ds->inv_mu[m];
+      th0 = ds->th0[m];
+      eps = ds->jeps;
+    }
     const double s = sum_partials(a.part + r_grad + (size_t)m * a.stride, nx, sh);
-    if (threadIdx.x == 0) ds->jgrad[m] = (a.alpha - 1.0) + 0.5 * a.inv_nv * s;
+    if (t == 0) {
+      const double g = (a.alpha - 1.0) + 0.5 * a.inv_nv * s;
+      if (kind == J_FIRST) ds->je0[m] = 0.5 * rho * rho * im + (a.alpha - 1.0) * th;
+      rho -= (kind == J_MID ? eps : 0.5 * eps) * g;
+      ds->rho[m] = rho;
+      if (kind == J_LAST) {
+        ds->je1[m] = 0.5 * rho * rho * im + (a.alpha - 1.0) * th;
+      } else {
+        th += eps * rho * im;
+        ds->th[m] = th;
+        ds->js[m] = (float)exp(0.5 * (th - th0));
+      }
+    }
   } else {
     // a reused force stage left its likelihood partials where the move's last one wrote them
     const double s = sum_partials(a.part + (ds->jreuse ? r_lik_move : r_lik), nz, sh);
-    if (threadIdx.x == 0) ds->jlik = s;
+    if (t == 0) {
+      if (kind == J_FIRST) {
+        ds->jlik0 = s;
+        ds->jreuse = 0;           // only the first gradient can reuse the move's force
+      } else {
+        ds->jlik1 = s;
+      }
+    }
   }
-  if (threadIdx.x == 0) {
+  if (kind != J_LAST) return;
+  if (t == 0) {
     __threadfence();
     s_last = atomicAdd(&ds->jdone, 1) == (int)gridDim.x - 1;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  if (threadIdx.x == 0) {
-    ds->jdone = 0;
-    ds->jreuse = 0;               // only the first gradient can reuse the move's force
+  if (t < 32) {
+    double e0 = 0.0, e1 = 0.0;
+    for (int i = t; i < a.n_bins; i += 32) {
+      e0 += ds->je0[i];
+      e1 += __ldcg(ds->je1 + i);
+    }
+    e0 = warp_sum(e0);
+    e1 = warp_sum(e1);
+    if (t == 0) {
+      ds->jdone = 0;
+      const double H0 = e0 + ds->jlik0, H1 = e1 + __ldcg(&ds->jlik1);
+      const double dH = H1 - H0;
+      ds->jH0 = H0;
+      ds->jH1 = H1;
+      ds->jdH = dH;
+      int acc = 0;
+      if (!isfinite(dH)) ds->status |= ST_NONFINITE;
+      else acc = ds->jlog_u < -dH;
+      ds->jaccepted = acc;
+      s_acc = acc;
+    }
   }
-  jump_update(a, kind, sh);
+  __syncthreads();
+  if (s_acc && t < a.n_bins) ds->P[t] = exp(ds->th[t]);
 }
 
 // ------------------------------------------------------------------ misc
@@ -482,7 +536,8 @@ __global__ void k_reduce_to(ScalarArgs a, int region, int nblk, double scale, do
   if (threadIdx.x == 0) out[q] = s * scale;
 }
 
-// chain record: P[n_bins], b[n_sub], nbar[n_sub], dH, accepted; slot rec_idx
+// End of a Gibbs iteration: the chain record P[n_bins], b[n_sub], nbar[n_sub], dH, accepted, and
+// the iteration counter.  Slot rec_idx
 // of chain (chain0 + blockIdx.y) in a buffer laid out [slot][chain][rec_len]
 __global__ void k_record(ScalarArgs a0, double* rec0, int rec_len, long long iter_stride, int chain0) {
   const ScalarArgs a = chain_args(a0, blockIdx.y);
@@ -500,7 +555,10 @@ __global__ void k_record(ScalarArgs a0, double* rec0, int rec_len, long long ite
     rec[a.n_bins + 2 * ns + 1] = (double)ds->accepted;
   }
   __syncthreads();
-  if (t == 0) ds->rec_idx += 1;
+  if (t == 0) {
+    ds->rec_idx += 1;
+    ds->iteration += 1;
+  }
 }
 
 __global__ void k_advance(DevState* ds) { ds[blockIdx.x].iteration += 1; }
@@ -521,23 +579,16 @@ __global__ void k_mstat(ScalarArgs a0, int region, int nblk, int final_) {
   }
 }
 
-void launch_move_begin(const ScalarArgs& a, int nch, cudaStream_t s) { k_move_begin<<<dim3(1, nch), MAXB, 0, s>>>(a); }
+void launch_move_begin(const ScalarArgs& a, int nch, cudaStream_t s) { k_move_begin<<<dim3(1, nch), 288, 0, s>>>(a); }
 void launch_move_end(const ScalarArgs& a, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz, int nch,
                      cudaStream_t s) {
-  k_move_sums<<<dim3(8, nch), 256, 0, s>>>(a, r_init, r_lik0, r_final, r_lik1, nx, nz);
-  k_move_end<<<dim3(1, nch), 32, 0, s>>>(a);
+  k_move_end<<<dim3(8, nch), 256, 0, s>>>(a, r_init, r_lik0, r_final, r_lik1, nx, nz);
 }
-void launch_power(const ScalarArgs& a, int region, int nx, int draw, int nch, cudaStream_t s) {
-  k_power<<<dim3(a.n_bins, nch), 256, 0, s>>>(a, region, nx, draw);
+void launch_power(const ScalarArgs& a, int region, int nx, int draw, int jump, int nch, cudaStream_t s) {
+  k_power<<<dim3(a.n_bins, nch), 320, 0, s>>>(a, region, nx, draw, jump);
 }
 void launch_bias_nbar(const ScalarArgs& a, int region, int nz, int nch, cudaStream_t s) {
-  k_bias_nbar<<<dim3(a.max_sub, nch), 256, 0, s>>>(a, region, nz);
-}
-void launch_abar(const ScalarArgs& a, int region, int nblk, int nch, cudaStream_t s) {
-  k_abar<<<dim3(1, nch), 256, 0, s>>>(a, region, nblk);
-}
-void launch_jump_begin(const ScalarArgs& a, int reuse, int nch, cudaStream_t s) {
-  k_jump_begin<<<dim3(1, nch), MAXB, 0, s>>>(a, reuse);
+  k_bias_nbar<<<dim3(a.max_sub, nch), 352, 0, s>>>(a, region, nz);
 }
 void launch_jump_step(const ScalarArgs& a, int r_grad, int nx, int r_lik, int r_lik_move, int nz, int kind,
                       int nch, cudaStream_t s) {

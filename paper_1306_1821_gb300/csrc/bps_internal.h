@@ -78,6 +78,7 @@ struct YzEntry {
   int tiles = 0;
 };
 bool yz_table(int N, int nch, int n_sm, YzEntry* out);
+// a and c of every voxel, and abar in the launch's last block
 void launch_rebuild(const Fields& fp, long long nv, int region, int blocks, int nch, cudaStream_t s);
 // Data check of one subsample; with `span` (N a multiple of 32) it also widens
 // the per-line support of R > 0 (Fields::span encoding).
@@ -105,16 +106,16 @@ struct ScalarArgs {
 void launch_move_begin(const ScalarArgs& a, int nch, cudaStream_t s);
 void launch_move_end(const ScalarArgs& a, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz, int nch,
                      cudaStream_t s);
-void launch_power(const ScalarArgs& a, int region, int nx, int draw, int nch, cudaStream_t s);
+// sigma of every bin, the P draw (draw = 1) and the start of the jump's HMC (jump = 1; 2: after an
+// accepted HMC move the jump's first gradient takes the move's last force stage)
+void launch_power(const ScalarArgs& a, int region, int nx, int draw, int jump, int nch, cudaStream_t s);
 void launch_bias_nbar(const ScalarArgs& a, int region, int nz, int nch, cudaStream_t s);
-void launch_abar(const ScalarArgs& a, int region, int nblk, int nch, cudaStream_t s);
-// reuse = 1: after an accepted HMC move the first gradient takes the move's last force stage
-void launch_jump_begin(const ScalarArgs& a, int reuse, int nch, cudaStream_t s);
 // reduce the jump gradient and likelihood partials, then the leapfrog update of `kind` (one launch)
 void launch_jump_step(const ScalarArgs& a, int r_grad, int nx, int r_lik, int r_lik_move, int nz, int kind,
                       int nch, cudaStream_t s);
 void launch_reduce_to(const ScalarArgs& a, int region, int nblk, int count, double scale, double* out_dev,
                       cudaStream_t s);
+// chain record, then the iteration counter
 void launch_record(const ScalarArgs& a, double* rec_dev, int rec_len, long long iter_stride, int chain0, int nch,
                    cudaStream_t s);
 void launch_advance(DevState* ds, int nch, cudaStream_t s);

@@ -1429,7 +1429,23 @@ __global__ void __launch_bounds__(256) k_rebuild(Fields fp0, long long nv, int r
   k.s = acc;
   k.c = -comp;
   double s = block_sum2<256>(k, reinterpret_cast<float*>(s_red));
-  if (threadIdx.x == 0) fp.part[region + blockIdx.x] = s;
+  // the last block to finish sums the blocks' partials, in a fixed order, into abar
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    fp.part[region + blockIdx.x] = s;
+    __threadfence();
+    s_last = atomicAdd(&ds->rdone, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double v = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) v += __ldcg(fp.part + region + i);
+  v = block_sum<256>(v, s_red);
+  if (threadIdx.x == 0) {
+    ds->abar = v * (1.0 / (double)nv);
+    ds->rdone = 0;
+  }
 }
 
 // Data check and compression: counts int32 -> uint16, R copied; per block the
