@@ -339,24 +339,33 @@ bps_status ds_read_bytes(bps_ctx* ctx, int ch, size_t off, void* dst, size_t n) 
   return BPS_OK;
 }
 
-// status words of all chains; cleared after reading
-bps_status check_status(bps_ctx* ctx) {
+constexpr size_t HOST_BUF = 64 * 1024;   // bytes of the pinned read-back buffer
+static_assert(sizeof(DevState) <= HOST_BUF / 2, "a chain state and a record fit the read-back buffer");
+
+// The chain's state after all queued work: one copy and one wait, instead of one of
+// each (8-10 us) per value that a call returns.  Valid until the next read-back.
+bps_status ds_snapshot(bps_ctx* ctx, int ch, const DevState** out) {
+  CK(cudaMemcpyAsync(ctx->host_buf, ctx->ds + ch, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  *out = reinterpret_cast<const DevState*>(ctx->host_buf);
+  return BPS_OK;
+}
+
+// Clears and reports the status words of chains [ch0, ch0 + n).
+bps_status report_status(bps_ctx* ctx, int ch0, const int* st, int n) {
   int any = 0;
-  for (int ch = 0; ch < ctx->batch; ++ch) {
-    int st = 0;
-    bps_status s = ds_read_bytes(ctx, ch, DS_OFF(status), &st, sizeof(int));
-    if (s != BPS_OK) return s;
-    if (st != 0) {
-      int zero = 0;
-      ds_write_bytes(ctx, ch, DS_OFF(status), &zero, sizeof(int));
-      any |= st;
-      if (st & ST_BADDATA) {
-        // a chain whose surveys were all invalid has none: only a valid commit
-        // writes the observed-voxel counts
-        double nobs0 = 0.0;
-        if (ds_read_bytes(ctx, ch, DS_OFF(nobs), &nobs0, sizeof(double)) == BPS_OK && !(nobs0 > 0.0))
-          ctx->have_data[ch] = 0;
-      }
+  for (int i = 0; i < n; ++i) {
+    if (st[i] == 0) continue;
+    const int s = st[i], ch = ch0 + i, zero = 0;   // st may lie in the read-back buffer
+    ds_write_bytes(ctx, ch, DS_OFF(status), &zero, sizeof(int));
+    any |= s;
+    if (s & ST_BADDATA) {
+      // a chain whose surveys were all invalid has none: only a valid commit
+      // writes the observed-voxel counts
+      double nobs0 = 0.0;
+      CK(cudaMemcpyAsync(&nobs0, ds_addr(ctx, ch, DS_OFF(nobs)), sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+      CK(cudaStreamSynchronize(ctx->stream));
+      if (!(nobs0 > 0.0)) ctx->have_data[ch] = 0;
     }
   }
   if (any & ST_BADDATA)
@@ -367,6 +376,27 @@ bps_status check_status(bps_ctx* ctx) {
   if (any & ST_NONFINITE) return fail(ctx, BPS_ENUMERIC, "non-finite energy difference; move rejected");
   if (any) return fail(ctx, BPS_ENUMERIC, "a scalar draw failed (no acceptance within the attempt bound or a non-positive sum)");
   return BPS_OK;
+}
+
+// The status words of all chains into dst (pinned), queued on the stream.
+bps_status queue_status(bps_ctx* ctx, int* dst) {
+  CK(cudaMemcpy2DAsync(dst, sizeof(int), ds_addr(ctx, 0, DS_OFF(status)), sizeof(DevState), sizeof(int), ctx->batch,
+                       cudaMemcpyDeviceToHost, ctx->stream));
+  return BPS_OK;
+}
+
+// status words of all chains; cleared after reading
+bps_status check_status(bps_ctx* ctx) {
+  std::vector<int> big;
+  int* st = reinterpret_cast<int*>(ctx->host_buf);
+  if ((size_t)ctx->batch * sizeof(int) > HOST_BUF) {
+    big.resize(ctx->batch);
+    st = big.data();
+  }
+  bps_status s = queue_status(ctx, st);
+  if (s != BPS_OK) return s;
+  CK(cudaStreamSynchronize(ctx->stream));
+  return report_status(ctx, 0, st, ctx->batch);
 }
 
 // ------------------------------------------------------------------ profiling
@@ -601,6 +631,10 @@ bps_status need_data(bps_ctx* ctx) {
   }
   return BPS_OK;
 }
+
+// Callers' half spectra are written by kernels as 8-byte elements; an array that
+// starts off an 8-byte boundary takes a copy.
+bool aligned8(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7) == 0; }
 
 bps_status copy_spec_out(bps_ctx* ctx, const float2* src, float* dst) {
   const size_t H1 = (size_t)ctx->N / 2 + 1;
@@ -995,7 +1029,7 @@ bps_status create_group(int grid_n, const std::vector<double>& box, const std::v
             alloc((void**)&ctx->part, (size_t)ctx->part_cstride * B * sizeof(double)) &&
             alloc((void**)&ctx->ds, sizeof(DevState) * B) &&
             (!ids.empty() || alloc((void**)&ctx->chain_dev, (size_t)ctx->chain_cap * rec_len * sizeof(double))) &&
-            cudaMallocHost((void**)&ctx->host_buf, 64 * 1024) == cudaSuccess;
+            cudaMallocHost((void**)&ctx->host_buf, HOST_BUF) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     free_all(ctx);
@@ -1271,17 +1305,14 @@ bps_status get_state_chain(bps_ctx* ctx, int ch, float* delta_dev, double* P, do
     ctx->pt.z_c2r(f, f.W, delta_dev, ctx->stream);
     LAUNCHED(ctx, 3);
   }
-  const int ns = ctx->nsub[ch];
-  if (P) st = ds_read_bytes(ctx, ch, DS_OFF(P), P, ctx->cfg.n_bins * sizeof(double));
-  if (st == BPS_OK && b) st = ds_read_bytes(ctx, ch, DS_OFF(b), b, ns * sizeof(double));
-  if (st == BPS_OK && nbar) st = ds_read_bytes(ctx, ch, DS_OFF(nbar), nbar, ns * sizeof(double));
-  if (st == BPS_OK && iteration) {
-    unsigned long long it = 0;
-    st = ds_read_bytes(ctx, ch, DS_OFF(iteration), &it, sizeof(it));
-    *iteration = it;
-  }
+  const DevState* ds = nullptr;
+  st = ds_snapshot(ctx, ch, &ds);
   if (st != BPS_OK) return st;
-  CK(cudaStreamSynchronize(ctx->stream));
+  const int ns = ctx->nsub[ch];
+  if (P) std::copy(ds->P, ds->P + ctx->cfg.n_bins, P);
+  if (b) std::copy(ds->b, ds->b + ns, b);
+  if (nbar) std::copy(ds->nbar, ds->nbar + ns, nbar);
+  if (iteration) *iteration = ds->iteration;
   return BPS_OK;
 }
 
@@ -1403,6 +1434,43 @@ bps_status run_iterations(bps_ctx* top, const std::vector<bps_ctx*>& groups, int
   }
   for (int i = 0; i < n_iter; ++i) CK(cudaGraphLaunch(top->graph, s));
   top->launches += (uint64_t)n_iter * top->graph_launches;
+  return BPS_OK;
+}
+
+// The end of a run: `n` record values from rec_dev into out (host) and the status
+// words of every chain of the groups, with one wait for all of them.  Records that
+// fit come through the pinned buffer (a copy to pageable memory waits by itself).
+bps_status read_back(bps_ctx* top, const std::vector<bps_ctx*>& groups, const double* rec_dev, size_t n, double* out) {
+  bps_ctx* ctx = top;
+  size_t chains = 0;
+  for (const bps_ctx* g : groups) chains += (size_t)g->batch;
+  const size_t rec_bytes = n * sizeof(double), st_bytes = chains * sizeof(int);
+  const bool pinned = rec_bytes + st_bytes <= HOST_BUF;
+  std::vector<int> own;
+  int* st = reinterpret_cast<int*>(reinterpret_cast<char*>(top->host_buf) + (pinned ? rec_bytes : 0));
+  if (!pinned) {
+    own.resize(chains);
+    st = own.data();
+  }
+  if (n)
+    CK(cudaMemcpyAsync(pinned ? top->host_buf : out, rec_dev, rec_bytes, cudaMemcpyDeviceToHost, top->stream));
+  size_t at = 0;
+  for (bps_ctx* g : groups) {
+    bps_status s = queue_status(g, st + at);
+    if (s != BPS_OK) return s;
+    at += (size_t)g->batch;
+  }
+  CK(cudaStreamSynchronize(top->stream));
+  if (n && pinned) std::memcpy(out, top->host_buf, rec_bytes);
+  at = 0;
+  for (bps_ctx* g : groups) {
+    bps_status s = report_status(g, 0, st + at, g->batch);
+    if (s != BPS_OK) {
+      top->err = g->err;
+      return s;
+    }
+    at += (size_t)g->batch;
+  }
   return BPS_OK;
 }
 
@@ -1618,11 +1686,15 @@ bps_status bps_get_state(bps_ctx* ctx, float* delta_dev, double* P, double* b, d
 
 bps_status bps_get_spectrum(bps_ctx* ctx, float* spec_dev) {
   if (!ctx || ctx->is_batch || !spec_dev) return fail(ctx, BPS_EINVAL, "null argument or batch context");
-  bps_status st;
-  int cur = current_buffer(ctx, 0, &st);
-  if (st != BPS_OK) return st;
-  st = copy_spec_out(ctx, ctx->dh[cur], spec_dev);
-  if (st != BPS_OK) return st;
+  if (aligned8(spec_dev)) {
+    launch_spec_out(fields_at(ctx, 0), reinterpret_cast<float2*>(spec_dev), ctx->zp, ctx->stream);
+    LAUNCHED(ctx, 1);
+  } else {
+    bps_status st;
+    const int cur = current_buffer(ctx, 0, &st);
+    if (st == BPS_OK) st = copy_spec_out(ctx, ctx->dh[cur], spec_dev);
+    if (st != BPS_OK) return st;
+  }
   CK(cudaStreamSynchronize(ctx->stream));
   return BPS_OK;
 }
@@ -1880,19 +1952,14 @@ bps_status bps_hmc_step(bps_ctx* ctx, bps_move_info* info) {
   if (st != BPS_OK) return st;
   st = hmc_move(ctx, true);
   if (st != BPS_OK) return st;
-  if (info) {
-    int acc = 0;
-    double dH = 0, eps = 0;
-    st = ds_read_bytes(ctx, 0, DS_OFF(accepted), &acc, sizeof(int));
-    if (st == BPS_OK) st = ds_read_bytes(ctx, 0, DS_OFF(dH), &dH, sizeof(double));
-    if (st == BPS_OK) st = ds_read_bytes(ctx, 0, DS_OFF(eps), &eps, sizeof(double));
-    if (st != BPS_OK) return st;
-    info->accepted = acc;
-    info->dH = dH;
-    info->eps = eps;
-    return check_status(ctx);
-  }
-  return BPS_OK;
+  if (!info) return BPS_OK;
+  const DevState* ds = nullptr;
+  st = ds_snapshot(ctx, 0, &ds);
+  if (st != BPS_OK) return st;
+  info->accepted = ds->accepted;
+  info->dH = ds->dH;
+  info->eps = ds->eps;
+  return report_status(ctx, 0, &ds->status, 1);
 }
 
 bps_status bps_adapt_step_size(bps_ctx* ctx, int n_rounds, int moves_per_round, double target,
@@ -1935,11 +2002,13 @@ bps_status bps_sample_power(bps_ctx* ctx, double* P_out, double* sigma_out) {
   if (st != BPS_OK) return st;
   st = power_stage(ctx, true, true);
   if (st != BPS_OK) return st;
-  if (P_out) st = ds_read_bytes(ctx, 0, DS_OFF(P), P_out, ctx->cfg.n_bins * sizeof(double));
-  if (st == BPS_OK && sigma_out) st = ds_read_bytes(ctx, 0, DS_OFF(sigma), sigma_out, ctx->cfg.n_bins * sizeof(double));
+  if (!P_out && !sigma_out) return BPS_OK;
+  const DevState* ds = nullptr;
+  st = ds_snapshot(ctx, 0, &ds);
   if (st != BPS_OK) return st;
-  if (P_out || sigma_out) return check_status(ctx);
-  return BPS_OK;
+  if (P_out) std::copy(ds->P, ds->P + ctx->cfg.n_bins, P_out);
+  if (sigma_out) std::copy(ds->sigma, ds->sigma + ctx->cfg.n_bins, sigma_out);
+  return report_status(ctx, 0, &ds->status, 1);
 }
 
 bps_status bps_sample_bias_norm(bps_ctx* ctx, double* b_out, double* nbar_out, double* sums_out) {
@@ -1948,17 +2017,15 @@ bps_status bps_sample_bias_norm(bps_ctx* ctx, double* b_out, double* nbar_out, d
   if (st != BPS_OK) return st;
   st = bias_stage(ctx, true);
   if (st != BPS_OK) return st;
+  if (!b_out && !nbar_out && !sums_out) return BPS_OK;
   const int ns = ctx->nsub[0];
-  if (b_out) st = ds_read_bytes(ctx, 0, DS_OFF(b), b_out, ns * sizeof(double));
-  if (st == BPS_OK && nbar_out) st = ds_read_bytes(ctx, 0, DS_OFF(nbar), nbar_out, ns * sizeof(double));
-  if (st == BPS_OK && sums_out) {
-    std::vector<double> tmp(3 * MAXS);
-    st = ds_read_bytes(ctx, 0, DS_OFF(sums), tmp.data(), tmp.size() * sizeof(double));
-    for (int i = 0; i < 3 * ns; ++i) sums_out[i] = tmp[i];
-  }
+  const DevState* ds = nullptr;
+  st = ds_snapshot(ctx, 0, &ds);
   if (st != BPS_OK) return st;
-  if (b_out || nbar_out || sums_out) return check_status(ctx);
-  return BPS_OK;
+  if (b_out) std::copy(ds->b, ds->b + ns, b_out);
+  if (nbar_out) std::copy(ds->nbar, ds->nbar + ns, nbar_out);
+  if (sums_out) std::copy(&ds->sums[0][0], &ds->sums[0][0] + 3 * ns, sums_out);
+  return report_status(ctx, 0, &ds->status, 1);
 }
 
 bps_status bps_jump(bps_ctx* ctx, bps_move_info* info) {
@@ -1969,19 +2036,14 @@ bps_status bps_jump(bps_ctx* ctx, bps_move_info* info) {
     return fail(ctx, BPS_EINVAL, "jump settings are not set");
   st = jump_stage(ctx, true);
   if (st != BPS_OK) return st;
-  if (info) {
-    int acc = 0;
-    double dH = 0, eps = 0;
-    st = ds_read_bytes(ctx, 0, DS_OFF(jaccepted), &acc, sizeof(int));
-    if (st == BPS_OK) st = ds_read_bytes(ctx, 0, DS_OFF(jdH), &dH, sizeof(double));
-    if (st == BPS_OK) st = ds_read_bytes(ctx, 0, DS_OFF(jeps), &eps, sizeof(double));
-    if (st != BPS_OK) return st;
-    info->accepted = acc;
-    info->dH = dH;
-    info->eps = eps;
-    return check_status(ctx);
-  }
-  return BPS_OK;
+  if (!info) return BPS_OK;
+  const DevState* ds = nullptr;
+  st = ds_snapshot(ctx, 0, &ds);
+  if (st != BPS_OK) return st;
+  info->accepted = ds->jaccepted;
+  info->dH = ds->jdH;
+  info->eps = ds->jeps;
+  return report_status(ctx, 0, &ds->status, 1);
 }
 
 bps_status bps_gibbs_iterate(bps_ctx* ctx, int n_iter, double* chain_out) {
@@ -1992,18 +2054,20 @@ bps_status bps_gibbs_iterate(bps_ctx* ctx, int n_iter, double* chain_out) {
   if (n_iter == 0) return BPS_OK;
   const int rec = ctx->cfg.n_bins + 2 * ctx->max_sub + 2;
   // the record buffer holds up to chain_cap iterations; longer runs go in pieces
-  int done = 0;
-  while (done < n_iter) {
+  for (int done = 0; done < n_iter;) {
     const int k = std::min(n_iter - done, ctx->chain_cap);
     st = run_iterations(ctx, {ctx}, k, ctx->chain_dev, rec, 1, ctx->cfg.jump != 0);
     if (st != BPS_OK) return st;
-    if (chain_out)
-      CK(cudaMemcpyAsync(chain_out + (size_t)done * rec, ctx->chain_dev, (size_t)k * rec * sizeof(double),
-                         cudaMemcpyDeviceToHost, ctx->stream));
     done += k;
+    if (done < n_iter || !chain_out) {
+      if (chain_out)
+        CK(cudaMemcpyAsync(chain_out + (size_t)(done - k) * rec, ctx->chain_dev, (size_t)k * rec * sizeof(double),
+                           cudaMemcpyDeviceToHost, ctx->stream));
+      continue;
+    }
+    return read_back(ctx, {ctx}, ctx->chain_dev, (size_t)k * rec, chain_out + (size_t)(done - k) * rec);
   }
-  CK(cudaStreamSynchronize(ctx->stream));
-  return check_status(ctx);
+  return read_back(ctx, {ctx}, nullptr, 0, nullptr);
 }
 
 bps_status bps_set_mass_scale(bps_ctx* ctx, int n_mass_bins, const double* scales) {
@@ -2148,10 +2212,14 @@ bps_status bps_fft_r2c(bps_ctx* ctx, const float* real_dev, float* spec_dev) {
   Fields f = fields_at(ctx, 0);
   ctx->pt.z_r2c(f, real_dev, ctx->W, ctx->stream);
   ctx->pt.y_fwd(f, BUF_W, 1, ctx->stream);
-  ctx->pt.x_fwd(f, BUF_W, ctx->W, 1, ctx->stream);
+  const bool direct = aligned8(spec_dev);
+  if (direct) ctx->pt.x_out(f, reinterpret_cast<float2*>(spec_dev), ctx->stream);
+  else ctx->pt.x_fwd(f, BUF_W, ctx->W, 1, ctx->stream);
   LAUNCHED(ctx, 3);
-  bps_status st = copy_spec_out(ctx, ctx->W, spec_dev);
-  if (st != BPS_OK) return st;
+  if (!direct) {
+    bps_status st = copy_spec_out(ctx, ctx->W, spec_dev);
+    if (st != BPS_OK) return st;
+  }
   CK(cudaStreamSynchronize(ctx->stream));
   return BPS_OK;
 }
@@ -2181,16 +2249,18 @@ bps_status bps_gradient(bps_ctx* ctx, float* grad_dev, double* energies) {
   ctx->pt.x_inv(f, -1, ctx->W, 1, s);
   bps_status sf = force_stage(ctx, f, region_offset(ctx, RG_LIK0), false, s);
   if (sf != BPS_OK) return sf;
-  ctx->pt.x_grad(f, ctx->W, region_offset(ctx, RG_GRAD), 1, s);
-  double* scratch = reinterpret_cast<double*>(ds_addr(ctx, 0, DS_OFF(scratch)));
-  launch_reduce_to(sa, region_offset(ctx, RG_GRAD), ctx->pt.x_tiles, 1, 0.5 / (double)ctx->nv, scratch, s);
-  launch_reduce_to(sa, region_offset(ctx, RG_LIK0), lik_tiles(ctx), 1, 1.0, scratch + 1, s);
-  LAUNCHED(ctx, 5);
-  st = copy_spec_out(ctx, ctx->W, grad_dev);
-  if (st != BPS_OK) return st;
-  if (energies) {
-    st = ds_read_bytes(ctx, 0, DS_OFF(scratch), energies, 2 * sizeof(double));
+  const bool direct = aligned8(grad_dev);
+  ctx->pt.x_grad(f, direct ? reinterpret_cast<float2*>(grad_dev) : ctx->W, direct, region_offset(ctx, RG_GRAD), s);
+  LAUNCHED(ctx, 3);
+  if (!direct) {
+    st = copy_spec_out(ctx, ctx->W, grad_dev);
     if (st != BPS_OK) return st;
+  }
+  if (energies) {
+    launch_gradient_energies(sa, region_offset(ctx, RG_GRAD), ctx->pt.x_tiles, region_offset(ctx, RG_LIK0), lik_tiles(ctx),
+                             s);
+    LAUNCHED(ctx, 1);
+    return ds_read_bytes(ctx, 0, DS_OFF(scratch), energies, 2 * sizeof(double));
   }
   CK(cudaStreamSynchronize(s));
   return BPS_OK;
@@ -2244,7 +2314,7 @@ bps_status bps_create_batch(int n_chains, const int* grid_n, const double* box_l
   top->chain_cap = 256;
   if (cudaMalloc((void**)&top->chain_dev, (size_t)top->chain_cap * n_chains * top->rec_len_all * sizeof(double)) !=
           cudaSuccess ||
-      cudaMallocHost((void**)&top->host_buf, 64 * 1024) != cudaSuccess) {
+      cudaMallocHost((void**)&top->host_buf, HOST_BUF) != cudaSuccess) {
     cudaGetLastError();
     bps_destroy(top);
     return fail(nullptr, BPS_ENOMEM, "device allocation failed");
@@ -2294,25 +2364,18 @@ bps_status bps_batch_gibbs_iterate(bps_ctx* batch, int n_iter, double* chain_out
   bps_ctx* ctx = batch;
   const int n_chains = (int)batch->chain_map.size();
   const int rec = batch->rec_len_all;
-  int done = 0;
-  while (done < n_iter) {
+  for (int done = 0; done < n_iter;) {
     const int k = std::min(n_iter - done, batch->chain_cap);
     bps_status st = run_iterations(batch, batch->groups, k, batch->chain_dev, rec, n_chains, batch->cfg.jump != 0);
     if (st != BPS_OK) return st;
-    if (chain_out)
-      CK(cudaMemcpyAsync(chain_out + (size_t)done * n_chains * rec, batch->chain_dev,
-                         (size_t)k * n_chains * rec * sizeof(double), cudaMemcpyDeviceToHost, batch->stream));
+    const size_t n = (size_t)k * n_chains * rec;
+    double* out = chain_out ? chain_out + (size_t)done * n_chains * rec : nullptr;
     done += k;
+    if (done < n_iter && out)
+      CK(cudaMemcpyAsync(out, batch->chain_dev, n * sizeof(double), cudaMemcpyDeviceToHost, batch->stream));
+    if (done == n_iter && out) return read_back(batch, batch->groups, batch->chain_dev, n, out);
   }
-  CK(cudaStreamSynchronize(batch->stream));
-  for (bps_ctx* g : batch->groups) {
-    bps_status st = check_status(g);
-    if (st != BPS_OK) {
-      batch->err = g->err;
-      return st;
-    }
-  }
-  return BPS_OK;
+  return read_back(batch, batch->groups, nullptr, 0, nullptr);
 }
 
 bps_status bps_mass_stats(bps_ctx* ctx, int n_moves, int n_mass_bins, double* out) {

@@ -529,11 +529,12 @@ __global__ void __launch_bounds__(256) k_jump_step(ScalarArgs a0, int r_grad, in
 }
 
 // ------------------------------------------------------------------ misc
-__global__ void k_reduce_to(ScalarArgs a, int region, int nblk, double scale, double* out) {
+// block 0: prior energy, block 1: likelihood energy of a gradient evaluation
+__global__ void k_gradient_energies(ScalarArgs a, int r_prior, int nx, int r_lik, int nz) {
   __shared__ double sh[32];
-  const int q = blockIdx.x;
-  const double s = sum_partials(a.part + region + (size_t)q * a.stride, nblk, sh);
-  if (threadIdx.x == 0) out[q] = s * scale;
+  const bool prior = blockIdx.x == 0;
+  const double s = sum_partials(a.part + (prior ? r_prior : r_lik), prior ? nx : nz, sh);
+  if (threadIdx.x == 0) a.ds->scratch[blockIdx.x] = prior ? s * (0.5 * a.inv_nv) : s;
 }
 
 // End of a Gibbs iteration: the chain record P[n_bins], b[n_sub], nbar[n_sub], dH, accepted, and
@@ -595,9 +596,8 @@ void launch_jump_step(const ScalarArgs& a, int r_grad, int nx, int r_lik, int r_
   k_jump_step<<<dim3(a.n_bins + (kind == J_MID ? 0 : 1), nch), 256, 0, s>>>(a, r_grad, nx, r_lik, r_lik_move, nz,
                                                                           kind);
 }
-void launch_reduce_to(const ScalarArgs& a, int region, int nblk, int count, double scale, double* out_dev,
-                      cudaStream_t s) {
-  k_reduce_to<<<count, 256, 0, s>>>(a, region, nblk, scale, out_dev);
+void launch_gradient_energies(const ScalarArgs& a, int r_prior, int nx, int r_lik, int nz, cudaStream_t s) {
+  k_gradient_energies<<<2, 256, 0, s>>>(a, r_prior, nx, r_lik, nz);
 }
 void launch_record(const ScalarArgs& a, double* rec_dev, int rec_len, long long iter_stride, int chain0, int nch,
                    cudaStream_t s) {

@@ -23,7 +23,10 @@ struct PassTable {
   void (*x_final)(const Fields&, int region, int nch, cudaStream_t);
   void (*x_inv)(const Fields&, int src_buf, float2* dst, int nch, cudaStream_t);   // src_buf -1: current state; dst NULL: W
   void (*x_fwd)(const Fields&, int src_buf, float2* dst, int nch, cudaStream_t);   // dst NULL: current state
-  void (*x_grad)(const Fields&, float2* dst, int region, int nch, cudaStream_t);
+  // one chain, into a caller's unpadded half spectrum [N][N][N/2+1] (x_grad: or a padded one): the
+  // gradient, and FFT_x(W)
+  void (*x_grad)(const Fields&, float2* dst, bool unpadded, int region, cudaStream_t);
+  void (*x_out)(const Fields&, float2* dst, cudaStream_t);
   void (*x_jinv)(const Fields&, int nch, cudaStream_t);
   void (*x_jgrad)(const Fields&, int region, int nch, cudaStream_t);
   void (*x_scale)(const Fields&, int nch, cudaStream_t);
@@ -113,8 +116,10 @@ void launch_bias_nbar(const ScalarArgs& a, int region, int nz, int nch, cudaStre
 // reduce the jump gradient and likelihood partials, then the leapfrog update of `kind` (one launch)
 void launch_jump_step(const ScalarArgs& a, int r_grad, int nx, int r_lik, int r_lik_move, int nz, int kind,
                       int nch, cudaStream_t s);
-void launch_reduce_to(const ScalarArgs& a, int region, int nblk, int count, double scale, double* out_dev,
-                      cudaStream_t s);
+// DevState::scratch[0] = prior energy from nx partials, scratch[1] = likelihood energy from nz (one chain)
+void launch_gradient_energies(const ScalarArgs& a, int r_prior, int nx, int r_lik, int nz, cudaStream_t s);
+// the chain's current half spectrum into a caller's unpadded one
+void launch_spec_out(const Fields& f, float2* dst, int zp, cudaStream_t s);
 // chain record, then the iteration counter
 void launch_record(const ScalarArgs& a, double* rec_dev, int rec_len, long long iter_stride, int chain0, int nch,
                    cudaStream_t s);

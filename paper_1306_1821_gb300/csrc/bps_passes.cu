@@ -47,6 +47,7 @@ struct XArgs {
   int first;
   int region;    // offset (doubles) of this launch's partial sums in Fields::part
   const float* amp = nullptr;   // X_AMP: amplitude of every |n|^2
+  int unpadded = 0;             // X_GRAD, X_FWD: dst is a caller's half spectrum [N][N][N/2+1]
 };
 
 struct ZArgs {
@@ -200,11 +201,16 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   const int jc = t / F;                       // row group of the Fourier (kx-) layout
   const bool act = jc < R2;
 
+  // element (kx = k, ky, kz) of this column in dst
+  auto dst_idx = [&](int k) -> long long {
+    return xa.unpadded ? ((long long)k * N + ky) * (C::H + 1) + kz : colo + (long long)k * T.rs;
+  };
+  (void)dst_idx;
   if constexpr (MODE == X_FWD) {
     if (act) {
       float2* out = xa.dst ? xa.dst : dsel(fp, cur);
 #pragma unroll
-      for (int d = 0; d < R1; ++d) out[colo + (long long)(jc + R2 * d) * T.rs] = v[d];
+      for (int d = 0; d < R1; ++d) out[dst_idx(jc + R2 * d)] = v[d];
     }
     return;
   }
@@ -360,7 +366,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
           g = make_float2(fmaf(x[d].x, il, v[d].x), fmaf(x[d].y, il, v[d].y));
           eP.add(wk * (x[d].x * x[d].x + x[d].y * x[d].y) * il);
         }
-        xa.dst[colo + (long long)k * T.rs] = g;
+        xa.dst[dst_idx(k)] = g;
       }
     }
     double sP = block_sum2<NT>(eP, reinterpret_cast<float*>(s_red));
@@ -1633,6 +1639,18 @@ __global__ void k_voxel_normals(uint64_t seed, uint64_t it, size_t n, float* out
   }
 }
 
+// The chain's current half spectrum into a caller's array without the pad column:
+// one warp per row, which reads the state index on the device (a 2D copy needs it on
+// the host first).
+__global__ void __launch_bounds__(256) k_spec_out(Fields fp, float2* __restrict__ dst, int zp) {
+  const int H1 = fp.grid_n / 2 + 1, lane = threadIdx.x & 31;
+  const long long row = blockIdx.x * 8LL + (threadIdx.x >> 5);
+  if (row >= (long long)fp.grid_n * fp.grid_n) return;
+  const float2* src = dsel(fp, fp.ds->cur) + row * zp;
+  float2* out = dst + row * H1;
+  for (int k = lane; k < H1; k += 32) out[k] = src[k];
+}
+
 // ------------------------------------------------------------------ launch tables
 template <int N>
 struct Launch {
@@ -1677,7 +1695,8 @@ static PassTable make_table() {
   T.x_final = [](const Fields& f, int region, int n, cudaStream_t s) { L::template x<X_FINAL>(f, XArgs{-1, nullptr, 0, region}, n, s); };
   T.x_inv = [](const Fields& f, int src, float2* dst, int n, cudaStream_t s) { L::template x<X_INV>(f, XArgs{src, dst, 0, -1}, n, s); };
   T.x_fwd = [](const Fields& f, int src, float2* dst, int n, cudaStream_t s) { L::template x<X_FWD>(f, XArgs{src, dst, 0, -1}, n, s); };
-  T.x_grad = [](const Fields& f, float2* dst, int region, int n, cudaStream_t s) { L::template x<X_GRAD>(f, XArgs{-1, dst, 0, region}, n, s); };
+  T.x_grad = [](const Fields& f, float2* dst, bool unpadded, int region, cudaStream_t s) { L::template x<X_GRAD>(f, XArgs{-1, dst, 0, region, nullptr, unpadded}, 1, s); };
+  T.x_out = [](const Fields& f, float2* dst, cudaStream_t s) { L::template x<X_FWD>(f, XArgs{BUF_W, dst, 0, -1, nullptr, 1}, 1, s); };
   T.x_jinv = [](const Fields& f, int n, cudaStream_t s) { L::template x<X_JINV>(f, XArgs{-1, nullptr, 0, -1}, n, s); };
   T.x_jgrad = [](const Fields& f, int region, int n, cudaStream_t s) { L::template x<X_JGRAD>(f, XArgs{-1, nullptr, 0, region}, n, s); };
   T.x_scale = [](const Fields& f, int n, cudaStream_t s) { L::template x<X_SCALE>(f, XArgs{-1, nullptr, 0, -1}, n, s); };
@@ -1823,6 +1842,9 @@ bool pass_table(int N, PassTable* out) {
   }
 }
 
+void launch_spec_out(const Fields& f, float2* dst, int zp, cudaStream_t s) {
+  k_spec_out<<<(unsigned)(((long long)f.grid_n * f.grid_n + 7) / 8), 256, 0, s>>>(f, dst, zp);
+}
 void launch_rebuild(const Fields& fp, long long nv, int region, int blocks, int nch, cudaStream_t s) {
   k_rebuild<<<dim3(blocks, nch), 256, 0, s>>>(fp, nv, region);
 }
