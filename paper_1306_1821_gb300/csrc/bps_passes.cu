@@ -126,7 +126,9 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   // per-warp bin sums as compensated FP32 pairs (sum, error): FP64 arithmetic is
   // scarce on this GPU, and each pair keeps the sum of the FP32 terms it was given
   // to about twice FP32 precision
-  __shared__ float s_wh[BINNED ? NW : 1][MAXB], s_wl[BINNED ? NW : 1][MAXB];
+  // (one set per column that a warp works on at a time: step (2) of the binned modes)
+  constexpr int LPC = N == 256 ? 32 : 16, NH = NW * (32 / LPC);
+  __shared__ float s_wh[BINNED ? NH : 1][MAXB], s_wl[BINNED ? NH : 1][MAXB];
 
   const int t = threadIdx.x;
   DevState* ds = fp.ds;
@@ -147,7 +149,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
     s_sms[i] = ds->sqrt_ms[i];
     s_js[i] = ds->js[i];
     if constexpr (BINNED) {
-      for (int w = 0; w < NW; ++w) {
+      for (int w = 0; w < NH; ++w) {
         s_wh[w][i] = 0.f;
         s_wl[w][i] = 0.f;
       }
@@ -289,9 +291,12 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
           xx = make_float2(0.f, 0.f);
           pp = make_float2(0.f, 0.f);
         }
+        // delta and p are next read one leapfrog step later, after three passes over W:
+        // written as streaming data (first to leave L2) they leave it to W.  256^3:
+        // 5119 -> 5001 us per Gibbs iteration; streaming loads of them cost 1%.
         const long long idx = colo + (long long)k * T.rs;
-        fp.ph[idx] = pp;
-        dst[idx] = xx;
+        __stcs(fp.ph + idx, pp);
+        __stcs(dst + idx, xx);
         v[d] = xx;
       }
       }
@@ -396,7 +401,12 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
     const float2* src = (MODE == X_INV && xa.src_buf >= 0) ? buf_ptr(fp, xa.src_buf) : dsel(fp, cur);
     if (act) {
 #pragma unroll
-      for (int d = 0; d < R1; ++d) v[d] = src[colo + (long long)(jc + R2 * d) * T.rs];
+      for (int d = 0; d < R1; ++d) {
+        const float2* p = src + colo + (long long)(jc + R2 * d) * T.rs;
+        // the jump reads delta again only after the force stage has gone over W twice: a
+        // streaming load leaves L2 to W (256^3: 5001 -> 4953 us per Gibbs iteration)
+        v[d] = MODE == X_JINV ? __ldcs(p) : *p;
+      }
       if constexpr (MODE == X_JINV) {
         // the jump's field scale by bin, the bins read from the context's map
 #pragma unroll
@@ -431,9 +441,11 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
     const int warp = t >> 5, lane = t & 31;
     // (1) every element's term into shared memory by (row kx, column f); the
     // bin factor s_m of the jump gradient is applied per bin at the end
-    // column-major with a row stride of N + 2 floats: the writes (16 columns x 2
-    // rows per warp) and the reads (32 lanes L rows apart) both avoid bank conflicts
-    constexpr int SE = N + 2;
+    // column-major with a column stride of N + 32 / F floats: the writes (F columns
+    // x 32 / F rows per warp) and the reads (lanes L rows apart; of two columns F / 2
+    // apart, which fall on different halves of the banks) both avoid conflicts
+    constexpr int SE = N + 32 / F;
+    static_assert(F * SE <= 2 * N * F, "the terms fit the exchange buffer");
     float* s_e = reinterpret_cast<float*>(s_ex);   // F * SE floats, free after the transform
     if (act) {
       float2 xv[R1];
@@ -458,26 +470,33 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
       }
     }
     __syncthreads();
-    // (2) one warp per column.  Lane q takes |nx| in [q L, q L + L) (both rows
-    // kx = |nx| and N - |nx|), in rising order, so its bins rise; consecutive
+    // (2) LPC lanes of a warp per column.  Lane q takes |nx| in [q L, q L + L) (both
+    // rows kx = |nx| and N - |nx|), in rising order, so its bins rise; consecutive
     // lanes follow each other.  A lane sums its elements into runs of equal
-    // bin: a run that starts and ends inside the lane holds a bin no other lane
-    // has and goes straight to the warp's bins; the lane's first and last runs
-    // are combined across the warp by segmented sums (the first runs and the
-    // last runs each form a bin-ordered sequence over the lanes).  Fixed order
-    // throughout: the sums are deterministic.
-    constexpr int HN = N / 2, L = (HN + 1 + 31) / 32;
+    // bin: a run that starts and ends inside the lane holds a bin no other lane of
+    // the column has and goes straight to the column's bins; the lane's first and
+    // last runs are combined across the lanes by segmented sums (the first runs
+    // and the last runs each form a bin-ordered sequence).  Fixed order throughout:
+    // the sums are deterministic.  The combination costs as much as a lane's few
+    // elements, so up to 128^3 two columns share it, half a warp each (the jump
+    // gradient of 32 chains of 96^3 111 -> 91 us, of 64^3 37 -> 29 us, at 128^3 13.9 -> 12.4 us);
+    // at 256^3 nine elements per lane and the second set of bins cost more than
+    // that (k-bin power 30 -> 37 us), and a column has the whole warp.
+    constexpr int HN = N / 2, L = (HN + 1 + LPC - 1) / LPC, CPW = 32 / LPC;
+    static_assert(F % CPW == 0, "columns of a warp");
     const int* thr = MASSBINS ? s_mthr : s_thr;
     const int nb = MASSBINS ? fp.n_mass : fp.n_bins;
     const float scl = MASSBINS ? scm : scb;
-    float* wh = s_wh[warp];
-    float* wl = s_wl[warp];
-    for (int col = warp; col < F; col += NW) {
+    const int part = lane / LPC, ql = lane % LPC;
+    float* wh = s_wh[CPW * warp + part];
+    float* wl = s_wl[CPW * warp + part];
+    for (int c0 = warp; c0 < F / CPW; c0 += NW) {
+      const int col = c0 + part * (F / CPW);
       const int nyc = sgn_n<N>(T.ky0 + col * T.dky), kzc = T.kz0 + col * T.dkz;
       const int n2c = nyc * nyc + kzc * kzc;
-      const int a0 = lane * L, a1 = min(a0 + L, HN + 1);
+      const int a0 = ql * L, a1 = min(a0 + L, HN + 1);
       int mf = -1, ml = -1, mc = -1, nxt = 0x7fffffff;
-      float vf = 0.f, vl = 0.f, vc = 0.f;   // FP32 runs; the warp's bins are compensated FP32 pairs
+      float vf = 0.f, vl = 0.f, vc = 0.f;   // FP32 runs; the column's bins are compensated FP32 pairs
       bool first_done = false;
       for (int a = a0; a < a1; ++a) {
         const int n2 = a * a + n2c;
@@ -516,19 +535,21 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
       for (int pass = 0; pass < 2; ++pass) {
         float vv = pass == 0 ? vf : vl;
         int mm2 = pass == 0 ? mf : ml;
+        if constexpr (LPC * L > HN + 1) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int pm = __shfl_up_sync(0xffffffffu, mm2, o);
-          if (mm2 < 0 && lane >= o) mm2 = pm;
+          for (int o = 1; o < LPC; o <<= 1) {
+            const int pm = __shfl_up_sync(0xffffffffu, mm2, o, LPC);
+            if (mm2 < 0 && ql >= o) mm2 = pm;
+          }
         }
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const float pv = __shfl_down_sync(0xffffffffu, vv, o);
-          const int pm = __shfl_down_sync(0xffffffffu, mm2, o);
-          if (lane + o < 32 && pm == mm2) vv += pv;
+        for (int o = 1; o < LPC; o <<= 1) {
+          const float pv = __shfl_down_sync(0xffffffffu, vv, o, LPC);
+          const int pm = __shfl_down_sync(0xffffffffu, mm2, o, LPC);
+          if (ql + o < LPC && pm == mm2) vv += pv;
         }
-        const int prev = __shfl_up_sync(0xffffffffu, mm2, 1);
-        if ((lane == 0 || prev != mm2) && mm2 >= 0) two_sum_add(wh[mm2], wl[mm2], vv);
+        const int prev = __shfl_up_sync(0xffffffffu, mm2, 1, LPC);
+        if ((ql == 0 || prev != mm2) && mm2 >= 0) two_sum_add(wh[mm2], wl[mm2], vv);
         __syncwarp();
       }
     }
@@ -536,7 +557,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
     for (int m = t; m < MAXB; m += NT) {
       TwoSumAcc acc;
 #pragma unroll
-      for (int w = 0; w < NW; ++w) {
+      for (int w = 0; w < NH; ++w) {
         acc.add(s_wh[w][m]);
         acc.add(s_wl[w][m]);
       }
