@@ -439,13 +439,13 @@ void prof_mark(bps_ctx* ctx, int k) {
 
 // ------------------------------------------------------------------ stages (all chains of a group)
 bps_status rebuild_chain(bps_ctx* ctx, int ch) {
-  launch_rebuild(fields_at(ctx, ch), ctx->nv, region_offset(ctx, RG_RB), ctx->rebuild_blocks, 1, ctx->stream);
+  launch_rebuild(fields_at(ctx, ch), ctx->nv, region_offset(ctx, RG_RB), ctx->rebuild_blocks, 0, 1, ctx->stream);
   LAUNCHED(ctx, 1);
   return BPS_OK;
 }
 
-bps_status rebuild_all(bps_ctx* ctx) {
-  launch_rebuild(fields(ctx), ctx->nv, region_offset(ctx, RG_RB), ctx->rebuild_blocks, ctx->batch, ctx->stream);
+bps_status rebuild_all(bps_ctx* ctx, bool advance) {
+  launch_rebuild(fields(ctx), ctx->nv, region_offset(ctx, RG_RB), ctx->rebuild_blocks, advance, ctx->batch, ctx->stream);
   LAUNCHED(ctx, 1);
   return BPS_OK;
 }
@@ -504,13 +504,8 @@ bps_status hmc_move(bps_ctx* ctx, bool advance) {
   }
   P.x_final(f, region_offset(ctx, RG_FINAL), B, s);
   launch_move_end(sa, region_offset(ctx, RG_INIT), region_offset(ctx, RG_LIK0), region_offset(ctx, RG_FINAL),
-                  region_offset(ctx, RG_LIK1), P.x_tiles, lik_tiles(ctx), B, s);
-  int n = 6 + L + (ctx->mnet ? 1 : 0);
-  if (advance) {
-    launch_advance(ctx->ds, B, s);
-    ++n;
-  }
-  LAUNCHED(ctx, n);
+                  region_offset(ctx, RG_LIK1), P.x_tiles, lik_tiles(ctx), advance ? 1 : 0, B, s);
+  LAUNCHED(ctx, 6 + L + (ctx->mnet ? 1 : 0));
   return BPS_OK;
 }
 
@@ -541,13 +536,7 @@ bps_status bias_stage(bps_ctx* ctx, bool advance) {
   ctx->pt.z_sums(f, region_offset(ctx, RG_SUMS), B, s);
   launch_bias_nbar(sa, region_offset(ctx, RG_SUMS), ctx->pt.z_tiles, B, s);
   LAUNCHED(ctx, 4);
-  bps_status st = rebuild_all(ctx);
-  if (st != BPS_OK) return st;
-  if (advance) {
-    launch_advance(ctx->ds, B, s);
-    LAUNCHED(ctx, 1);
-  }
-  return BPS_OK;
+  return rebuild_all(ctx, advance);
 }
 
 // force evaluation of the jump at the current theta (scales js on the device)

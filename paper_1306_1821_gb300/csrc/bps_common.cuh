@@ -14,6 +14,14 @@ constexpr int MAXS = 16;   // maximum number of galaxy subsamples
 constexpr int FWD = -1;    // exp(-2 pi i jk/N): forward transform (App. C.1, C_hat = 1)
 constexpr int INV = +1;    // exp(+2 pi i jk/N): inverse transform (unnormalised here)
 
+// ---------------------------------------------------------------- launch order
+// Every kernel of a chain's stages is launched as a programmatic dependent of the
+// one before it (launch_dep, bps_internal.h): it may be brought onto the GPU while
+// that one drains, and does so here until it has completed and its writes are
+// visible.  All threads call this before they touch anything but the twiddle table
+// (written once at creation) or return.  No kernel triggers its dependents early.
+__device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- complex
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }

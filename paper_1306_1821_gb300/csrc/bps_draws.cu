@@ -40,6 +40,7 @@ __device__ double sum_partials(const double* p, int n, double* sh) {
 // Per-bin tables of the move and its scalars: two warps per table column (a
 // division and a square root each), one for the step size and the Metropolis draw.
 __global__ void __launch_bounds__(288) k_move_begin(ScalarArgs a0) {
+  await_previous();
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   DevState* ds = a.ds;
   const int t = threadIdx.x & 63, role = threadIdx.x >> 6;
@@ -75,7 +76,9 @@ __global__ void __launch_bounds__(288) k_move_begin(ScalarArgs a0) {
 // L1, G0, G1 (the kinetic, prior and likelihood energies at the start and the
 // end, and the two force norms of the leapfrog energy identity).  The last block
 // to finish takes the Metropolis decision.
-__global__ void k_move_end(ScalarArgs a0, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz) {
+__global__ void k_move_end(ScalarArgs a0, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz,
+                           int advance) {
+  await_previous();
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   __shared__ double sh[32];
   DevState* ds = a.ds;
@@ -134,6 +137,7 @@ __global__ void k_move_end(ScalarArgs a0, int r_init, int r_lik0, int r_final, i
       ds->n_accepted += 1;
     }
     ds->n_moves += 1;
+    if (advance) ds->iteration += 1;
   }
 }
 
@@ -187,6 +191,7 @@ __device__ double gamma_mt(double shape, uint64_t seed, uint64_t it, int m, int*
 // jump = 2: the jump directly follows this iteration's HMC move, so after an accepted
 // move its first gradient can take the move's last force.
 __global__ void __launch_bounds__(320) k_power(ScalarArgs a0, int region, int nx, int draw, int jump) {
+  await_previous();
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   __shared__ double sh[32];
   __shared__ double s_gamma, s_z, s_sigma, s_P;
@@ -332,6 +337,7 @@ __device__ double gig_draw(double p, double A, double B, const double* lu, const
 // iteration, ST_NBAR, j): word 0 gives u, word 1 the second uniform).
 // 66-75 us a launch with the section search and serial attempts, now 17-20 us.
 __global__ void __launch_bounds__(352) k_bias_nbar(ScalarArgs a0, int region, int nz) {
+  await_previous();
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   __shared__ double sh[3][8];
   __shared__ double s_S[3], s_z, s_lu[MAX_ATTEMPTS], s_u[MAX_ATTEMPTS], s_w[MAX_ATTEMPTS];
@@ -454,6 +460,7 @@ __global__ void k_commit_data(DevState* ds0, const double* part0, long long cstr
 // its last block, now 5.9 us.
 __global__ void __launch_bounds__(256) k_jump_step(ScalarArgs a0, int r_grad, int nx, int r_lik, int r_lik_move, int nz,
                                                    int kind) {
+  await_previous();
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   __shared__ double sh[32];
   __shared__ int s_last, s_acc;
@@ -531,6 +538,7 @@ __global__ void __launch_bounds__(256) k_jump_step(ScalarArgs a0, int r_grad, in
 // ------------------------------------------------------------------ misc
 // block 0: prior energy, block 1: likelihood energy of a gradient evaluation
 __global__ void k_gradient_energies(ScalarArgs a, int r_prior, int nx, int r_lik, int nz) {
+  await_previous();
   __shared__ double sh[32];
   const bool prior = blockIdx.x == 0;
   const double s = sum_partials(a.part + (prior ? r_prior : r_lik), prior ? nx : nz, sh);
@@ -541,6 +549,7 @@ __global__ void k_gradient_energies(ScalarArgs a, int r_prior, int nx, int r_lik
 // the iteration counter.  Slot rec_idx
 // of chain (chain0 + blockIdx.y) in a buffer laid out [slot][chain][rec_len]
 __global__ void k_record(ScalarArgs a0, double* rec0, int rec_len, long long iter_stride, int chain0) {
+  await_previous();
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   DevState* ds = a.ds;
   const int t = threadIdx.x;
@@ -562,14 +571,21 @@ __global__ void k_record(ScalarArgs a0, double* rec0, int rec_len, long long ite
   }
 }
 
-__global__ void k_advance(DevState* ds) { ds[blockIdx.x].iteration += 1; }
+__global__ void k_advance(DevState* ds) {
+  await_previous();
+  ds[blockIdx.x].iteration += 1;
+}
 
-__global__ void k_reset_rec(DevState* ds) { ds[blockIdx.x].rec_idx = 0; }
+__global__ void k_reset_rec(DevState* ds) {
+  await_previous();
+  ds[blockIdx.x].rec_idx = 0;
+}
 
 __global__ void k_zero_dc(float2* spec) { spec[0] = make_float2(0.f, 0.f); }
 
 // block j of chain blockIdx.y: sum of the per-tile partials of mass bin j
 __global__ void k_mstat(ScalarArgs a0, int region, int nblk, int final_) {
+  await_previous();
   const ScalarArgs a = chain_args(a0, blockIdx.y);
   __shared__ double sh[32];
   const int j = blockIdx.x;
@@ -580,38 +596,40 @@ __global__ void k_mstat(ScalarArgs a0, int region, int nblk, int final_) {
   }
 }
 
-void launch_move_begin(const ScalarArgs& a, int nch, cudaStream_t s) { k_move_begin<<<dim3(1, nch), 288, 0, s>>>(a); }
-void launch_move_end(const ScalarArgs& a, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz, int nch,
-                     cudaStream_t s) {
-  k_move_end<<<dim3(8, nch), 256, 0, s>>>(a, r_init, r_lik0, r_final, r_lik1, nx, nz);
+void launch_move_begin(const ScalarArgs& a, int nch, cudaStream_t s) {
+  launch_dep(k_move_begin, dim3(1, nch), dim3(288), 0, s, a);
+}
+void launch_move_end(const ScalarArgs& a, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz, int advance,
+                     int nch, cudaStream_t s) {
+  launch_dep(k_move_end, dim3(8, nch), dim3(256), 0, s, a, r_init, r_lik0, r_final, r_lik1, nx, nz, advance);
 }
 void launch_power(const ScalarArgs& a, int region, int nx, int draw, int jump, int nch, cudaStream_t s) {
-  k_power<<<dim3(a.n_bins, nch), 320, 0, s>>>(a, region, nx, draw, jump);
+  launch_dep(k_power, dim3(a.n_bins, nch), dim3(320), 0, s, a, region, nx, draw, jump);
 }
 void launch_bias_nbar(const ScalarArgs& a, int region, int nz, int nch, cudaStream_t s) {
-  k_bias_nbar<<<dim3(a.max_sub, nch), 352, 0, s>>>(a, region, nz);
+  launch_dep(k_bias_nbar, dim3(a.max_sub, nch), dim3(352), 0, s, a, region, nz);
 }
 void launch_jump_step(const ScalarArgs& a, int r_grad, int nx, int r_lik, int r_lik_move, int nz, int kind,
                       int nch, cudaStream_t s) {
-  k_jump_step<<<dim3(a.n_bins + (kind == J_MID ? 0 : 1), nch), 256, 0, s>>>(a, r_grad, nx, r_lik, r_lik_move, nz,
-                                                                          kind);
+  launch_dep(k_jump_step, dim3(a.n_bins + (kind == J_MID ? 0 : 1), nch), dim3(256), 0, s, a, r_grad, nx, r_lik,
+             r_lik_move, nz, kind);
 }
 void launch_gradient_energies(const ScalarArgs& a, int r_prior, int nx, int r_lik, int nz, cudaStream_t s) {
-  k_gradient_energies<<<2, 256, 0, s>>>(a, r_prior, nx, r_lik, nz);
+  launch_dep(k_gradient_energies, dim3(2), dim3(256), 0, s, a, r_prior, nx, r_lik, nz);
 }
 void launch_record(const ScalarArgs& a, double* rec_dev, int rec_len, long long iter_stride, int chain0, int nch,
                    cudaStream_t s) {
-  k_record<<<dim3(1, nch), MAXB, 0, s>>>(a, rec_dev, rec_len, iter_stride, chain0);
+  launch_dep(k_record, dim3(1, nch), dim3(MAXB), 0, s, a, rec_dev, rec_len, iter_stride, chain0);
 }
-void launch_advance(DevState* ds, int nch, cudaStream_t s) { k_advance<<<nch, 1, 0, s>>>(ds); }
+void launch_advance(DevState* ds, int nch, cudaStream_t s) { launch_dep(k_advance, dim3(nch), dim3(1), 0, s, ds); }
 void launch_commit_data(DevState* ds, const double* part, long long cstride, int nblk, int slot, int nch,
                         cudaStream_t s) {
   k_commit_data<<<nch, 1024, 0, s>>>(ds, part, cstride, nblk, slot);
 }
-void launch_reset_rec(DevState* ds, int nch, cudaStream_t s) { k_reset_rec<<<nch, 1, 0, s>>>(ds); }
+void launch_reset_rec(DevState* ds, int nch, cudaStream_t s) { launch_dep(k_reset_rec, dim3(nch), dim3(1), 0, s, ds); }
 void launch_zero_dc(float2* spec, cudaStream_t s) { k_zero_dc<<<1, 1, 0, s>>>(spec); }
 void launch_mstat(const ScalarArgs& a, int region, int nblk, int n_mass, int final_, int nch, cudaStream_t s) {
-  k_mstat<<<dim3(n_mass, nch), 256, 0, s>>>(a, region, nblk, final_);
+  launch_dep(k_mstat, dim3(n_mass, nch), dim3(256), 0, s, a, region, nblk, final_);
 }
 
 
@@ -620,6 +638,7 @@ void launch_mstat(const ScalarArgs& a, int region, int nblk, int n_mass, int fin
 // correlation matrices of P, b and Nbar), one FP64 accumulation per Gibbs
 // iteration, in a fixed order.
 __global__ void k_param_moments(ScalarArgs a, double* acc) {
+  await_previous();
   const DevState* ds = a.ds;
   const int nb = a.n_bins, ns = ds->nsub, D = nb + 2 * ns;
   __shared__ double x[MAXB + 2 * MAXS];
@@ -646,7 +665,7 @@ void launch_moments_finish(const double* mom, long long nv, double n, double* me
 }
 
 void launch_param_moments(const ScalarArgs& a, double* acc, cudaStream_t s) {
-  k_param_moments<<<1, 256, 0, s>>>(a, acc);
+  launch_dep(k_param_moments, dim3(1), dim3(256), 0, s, a, acc);
 }
 
 // ------------------------------------------------------------------ failure detection

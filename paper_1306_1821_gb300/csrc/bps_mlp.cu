@@ -431,6 +431,7 @@ namespace {
 // then s_j = exp(clamp(y_j)) into the chain's mass scales.  A matrix-vector
 // product per layer (at most 512 x 512): FP32 FMAs over coalesced weight rows.
 __global__ void __launch_bounds__(256) k_mass_net(ScalarArgs a, const MassNet* __restrict__ m) {
+  await_previous();
   DevState* ds = a.ds + blockIdx.y;
   __shared__ float h[2][MLP_MAX_WIDTH];
   const int t = threadIdx.x, nb = a.n_bins;
@@ -469,7 +470,7 @@ bps_status massnet_create(const bps_mlp* net, const float* mean, const float* sd
 void massnet_destroy(MassNet* m) { cudaFree(m); }
 
 void launch_mass_net(const ScalarArgs& a, const MassNet* m, int nch, cudaStream_t s) {
-  k_mass_net<<<dim3(1, nch), 256, 0, s>>>(a, m);
+  launch_dep(k_mass_net, dim3(1, nch), dim3(256), 0, s, a, m);
 }
 
 }  // namespace bps

@@ -132,13 +132,14 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
 
   const int t = threadIdx.x;
   DevState* ds = fp.ds;
+  load_twiddles<N>(s_tw, fp.tw, t, NT);
+  await_previous();
   if constexpr (MODE == X_SCALE) {
     if (!ds->jaccepted) return;   // uniform across the grid
   }
   if constexpr (MODE == X_JINV) {
     if (ds->jreuse) return;       // W already holds this force stage's input (uniform)
   }
-  load_twiddles<N>(s_tw, fp.tw, t, NT);
   for (int i = t; i < MAXB; i += NT) {
     s_thr[i] = ds->thr[i];
     s_mthr[i] = ds->mthr[i];
@@ -608,6 +609,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, (XTma<N, SD, SP>::MIN_BLOCKS))
   const int id = tile_id<N>();
   const Tile<N> T = tile_x<N>(id);
   const bool staged = id < N * C::ZB;
+  await_previous();
   const int cur = ds->cur;
   const int sbuf = xa.first ? cur : 1 - cur;
   if (staged && t == 0) {
@@ -757,6 +759,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, BPS_XLEAP_MIN_BLOCKS)
   const int id = tile_id<N>();
   const Tile<N> T = tile_x<N>(id);
   const bool staged = id < N * C::ZB;
+  await_previous();
   const int cur = ds->cur;
   const int sbuf = xa.first ? cur : 1 - cur;
   const CUtensorMap* dmap = sbuf ? &maps.d1q : &maps.d0q;
@@ -907,6 +910,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, BPS_XLEAP_MIN_BLOCKS)
 template <int N, int DIR>
 __global__ void __launch_bounds__(Cfg<N>::NT, BPS_YPASS_MIN_BLOCKS) k_ypass(Fields fp0, int buf) {
   const Fields fp = at_chain(fp0, blockIdx.y);
+  await_previous();
   if (buf == BUF_W && fp.ds->jreuse) return;   // force stage reused by the jump (uniform)
   using C = Cfg<N>;
   constexpr int F = C::F, R1 = C::R1, R2 = C::R2, NT = C::NT;
@@ -978,6 +982,7 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
   const int t = threadIdx.x;
   DevState* ds = fp.ds;
+  await_previous();
   if constexpr (MODE == Z_GRAD) {
     if (ds->jreuse) return;       // force stage reused by the jump (uniform)
   }
@@ -1284,6 +1289,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, BPS_XLEAP_MIN_BLOCKS)
   const int id = tile_id<N>();
   const Tile<N> T = tile_x<N>(id);
   const bool staged = id < N * C::ZB;
+  await_previous();
   const int cur = ds->cur;
   const int sbuf = xa.first ? cur : 1 - cur;
   const float2* src = dsel(fp, sbuf);
@@ -1405,11 +1411,12 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float x) {
 // the counts are zero wherever R = 0 (checked by set_data), so no mask is needed.
 // With per-line supports only the voxels inside them are computed: outside,
 // a = c = 0, which the data upload wrote once.
-__global__ void __launch_bounds__(256) k_rebuild(Fields fp0, long long nv, int region) {
+__global__ void __launch_bounds__(256) k_rebuild(Fields fp0, long long nv, int region, int advance) {
   const Fields fp = at_chain(fp0, blockIdx.y);
   __shared__ float s_a[MAXS], s_b[MAXS], s_bn[MAXS];
   __shared__ double s_red[32];
   DevState* ds = fp.ds;
+  await_previous();
   const int nsub = ds->nsub;
   if (threadIdx.x < nsub) {
     const double b = ds->b[threadIdx.x], nb = ds->nbar[threadIdx.x];
@@ -1472,6 +1479,7 @@ __global__ void __launch_bounds__(256) k_rebuild(Fields fp0, long long nv, int r
   if (threadIdx.x == 0) {
     ds->abar = v * (1.0 / (double)nv);
     ds->rdone = 0;
+    if (advance) ds->iteration += 1;
   }
 }
 
@@ -1666,6 +1674,7 @@ __global__ void k_voxel_normals(uint64_t seed, uint64_t it, size_t n, float* out
 __global__ void __launch_bounds__(256) k_spec_out(Fields fp, float2* __restrict__ dst, int zp) {
   const int H1 = fp.grid_n / 2 + 1, lane = threadIdx.x & 31;
   const long long row = blockIdx.x * 8LL + (threadIdx.x >> 5);
+  await_previous();
   if (row >= (long long)fp.grid_n * fp.grid_n) return;
   const float2* src = dsel(fp, fp.ds->cur) + row * zp;
   float2* out = dst + row * H1;
@@ -1678,15 +1687,15 @@ struct Launch {
   using C = Cfg<N>;
   template <int M>
   static void x(const Fields& fp, const XArgs& xa, int nch, cudaStream_t s) {
-    k_xpass<N, M><<<dim3(C::TILES, nch), C::NT, 0, s>>>(fp, xa);
+    launch_dep(k_xpass<N, M>, dim3(C::TILES, nch), dim3(C::NT), 0, s, fp, xa);
   }
   template <int D>
   static void y(const Fields& fp, int buf, int nch, cudaStream_t s) {
-    k_ypass<N, D><<<dim3(C::TILES, nch), C::NT, 0, s>>>(fp, buf);
+    launch_dep(k_ypass<N, D>, dim3(C::TILES, nch), dim3(C::NT), 0, s, fp, buf);
   }
   template <int M, int LP = C::LP>
   static void z(const Fields& fp, const ZArgs& za, int nch, cudaStream_t s) {
-    k_zpass<N, M, LP><<<dim3(N * N / (2 * LP), nch), LP * C::RMAX, ZSmem<N, M, LP>::BYTES, s>>>(fp, za);
+    launch_dep(k_zpass<N, M, LP>, dim3(N * N / (2 * LP), nch), dim3(LP * C::RMAX), ZSmem<N, M, LP>::BYTES, s, fp, za);
   }
   template <int M, int LP = C::LP>
   static void zattr() {
@@ -1746,8 +1755,8 @@ static PassTable make_table() {
 // ---------------------------------------------------------------- TMA x pass: maps and launch
 template <int N, int SD, int SP>
 void launch_xleap_tma(const Fields& f, const XMaps& m, int first, int nch, cudaStream_t s) {
-  k_xleap_tma<N, SD, SP><<<dim3(Cfg<N>::TILES, nch), Cfg<N>::NT, XTma<N, SD, SP>::SMEM, s>>>(
-      f, XArgs{-1, nullptr, first, -1}, m);
+  launch_dep(k_xleap_tma<N, SD, SP>, dim3(Cfg<N>::TILES, nch), dim3(Cfg<N>::NT), XTma<N, SD, SP>::SMEM, s, f,
+             XArgs{-1, nullptr, first, -1}, m);
 }
 
 template <int N, int SD, int SP>
@@ -1762,8 +1771,8 @@ XLeapTma xleap_entry() {
 
 template <int N, bool TMA>
 void launch_xleap_ring(const Fields& f, const XMaps& m, int first, int nch, cudaStream_t s) {
-  k_xleap_ring<N, TMA><<<dim3(Cfg<N>::TILES, nch), Cfg<N>::NT, XRing<N>::SMEM, s>>>(f, XArgs{-1, nullptr, first, -1},
-                                                                                      m);
+  launch_dep(k_xleap_ring<N, TMA>, dim3(Cfg<N>::TILES, nch), dim3(Cfg<N>::NT), XRing<N>::SMEM, s, f,
+             XArgs{-1, nullptr, first, -1}, m);
 }
 
 template <int N, bool TMA>
@@ -1778,7 +1787,8 @@ XLeapTma xleap_ring_entry() {
 
 template <int N>
 void launch_xleap_wring(const Fields& f, const XMaps& m, int first, int nch, cudaStream_t s) {
-  k_xleap_wring<N><<<dim3(Cfg<N>::TILES, nch), Cfg<N>::NT, XRing<N>::SMEM, s>>>(f, XArgs{-1, nullptr, first, -1}, m);
+  launch_dep(k_xleap_wring<N>, dim3(Cfg<N>::TILES, nch), dim3(Cfg<N>::NT), XRing<N>::SMEM, s, f,
+             XArgs{-1, nullptr, first, -1}, m);
 }
 
 template <int N>
@@ -1864,10 +1874,10 @@ bool pass_table(int N, PassTable* out) {
 }
 
 void launch_spec_out(const Fields& f, float2* dst, int zp, cudaStream_t s) {
-  k_spec_out<<<(unsigned)(((long long)f.grid_n * f.grid_n + 7) / 8), 256, 0, s>>>(f, dst, zp);
+  launch_dep(k_spec_out, dim3((unsigned)(((long long)f.grid_n * f.grid_n + 7) / 8)), dim3(256), 0, s, f, dst, zp);
 }
-void launch_rebuild(const Fields& fp, long long nv, int region, int blocks, int nch, cudaStream_t s) {
-  k_rebuild<<<dim3(blocks, nch), 256, 0, s>>>(fp, nv, region);
+void launch_rebuild(const Fields& fp, long long nv, int region, int blocks, int advance, int nch, cudaStream_t s) {
+  launch_dep(k_rebuild, dim3(blocks, nch), dim3(256), 0, s, fp, nv, region, advance);
 }
 void launch_data(const int32_t* cin, const float* rin, uint16_t* cout, float* rout, long long nv, double* part,
                  int stride, int blocks, int2* span, int n_grid, cudaStream_t s) {

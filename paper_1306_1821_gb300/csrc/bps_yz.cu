@@ -75,6 +75,12 @@ __global__ void __launch_bounds__(YZ<N, NW>::NT, YZ<N, NW>::MIN_BLOCKS) k_yzpass
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int plane = (int)blockIdx.x;
   float2* Wp = fp.W + (long long)plane * N * ZP;
+  for (int i = t; i < N; i += NT) {
+    tw[i] = fp.tw[i];
+    twa[i] = fp.tw[(i / A) * (i % A)];
+    twb[i] = fp.tw[(i / B) * (i % B)];
+  }
+  await_previous();
   // the first task's loads of the inverse y transform go out before anything waits
   // (a plane without support, which does not need them, is rare)
   float2 v0[B];
@@ -97,11 +103,6 @@ __global__ void __launch_bounds__(YZ<N, NW>::NT, YZ<N, NW>::MIN_BLOCKS) k_yzpass
     s_lo[i] = lo;
     s_hi[i] = hi;
     mine |= hi > lo;
-  }
-  for (int i = t; i < N; i += NT) {
-    tw[i] = fp.tw[i];
-    twa[i] = fp.tw[(i / A) * (i % A)];
-    twb[i] = fp.tw[(i / B) * (i % B)];
   }
   if (!__syncthreads_or(mine)) {
     // a plane without support has g = 0 on every line: a zero force, W not read
@@ -304,7 +305,7 @@ __global__ void __launch_bounds__(YZ<N, NW>::NT, YZ<N, NW>::MIN_BLOCKS) k_yzpass
 
 template <int N, int NW>
 void launch_yz(const Fields& f, int region, int nch, cudaStream_t s) {
-  k_yzpass<N, NW><<<dim3(N, nch), YZ<N, NW>::NT, YZ<N, NW>::BYTES, s>>>(f, region);
+  launch_dep(k_yzpass<N, NW>, dim3(N, nch), dim3(YZ<N, NW>::NT), YZ<N, NW>::BYTES, s, f, region);
 }
 
 template <int N, int NW>
