@@ -106,9 +106,23 @@ __device__ __forceinline__ const float2* buf_ptr(const Fields& fp, int b) {
 #define BPS_YPASS_MIN_BLOCKS 4
 #endif
 
+// Whether X_INIT, X_FINAL and X_GRAD work through the column in parts, three blocks
+// per SM, as the leapfrog pass does, or on the whole column (104-119 registers, two
+// blocks).  Parts win where many tiles wait for HBM: 256^3 74 -> 68, 66 -> 55 and 57 -> 48
+// us, 32 chains of 96^3 X_FINAL 174 -> 126 us.  One 128^3 grid fits L2 and has barely
+// more tiles than the SMs hold: 17 -> 20 us, so it keeps whole columns, as do the
+// smaller power-of-two grids.
+template <int N>
+struct XParts {
+  static constexpr bool value = N == 256 || N == 96;
+};
+
 // ------------------------------------------------------------------ x pass
 template <int N, int MODE>
-__global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG ? BPS_XLEAP_MIN_BLOCKS
+__global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG || MODE == X_AMP ||
+                                                      ((MODE == X_INIT || MODE == X_FINAL || MODE == X_GRAD) &&
+                                                       XParts<N>::value)
+                                                  ? BPS_XLEAP_MIN_BLOCKS
                                               : MODE == X_JINV  ? BPS_XJINV_MIN_BLOCKS
                                               : MODE == X_JGRAD ? BPS_XJGRAD_MIN_BLOCKS
                                                                 : BPS_XPASS_MIN_BLOCKS)
@@ -171,6 +185,11 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   const float scb = bin_scale(fp.n_bins, N), scm = bin_scale(fp.n_mass, N);
 
   float2 v[C::RMAX];
+  // modes that update or reduce the column against delta and p work through it in
+  // parts: the loads of a part in flight together, at a fraction of the registers
+  // of a whole column
+  constexpr bool WHOLE = (MODE == X_INIT || MODE == X_FINAL || MODE == X_GRAD) && !XParts<N>::value;
+  constexpr int PART = WHOLE ? R1 : R1 / BPS_XLEAP_CHUNKS > 0 ? R1 / BPS_XLEAP_CHUNKS : 1;
   auto mode_bin = [&](int k, float& il, float& im, float& sm) -> int {
     const int nx = sgn_n<N>(k);
     const int n2 = nx * nx + n2yz;
@@ -221,21 +240,24 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   if constexpr (MODE == X_INIT) {
     // momentum p = sqrt(M_k) FFT(xi); kinetic energy (1/2N^3) sum w |p|^2 / M
     TwoSumAcc eK, eP;
-    float2 x[R1];
     if (act) {
 #pragma unroll
-      for (int d = 0; d < R1; ++d) x[d] = dsel(fp, cur)[colo + (long long)(jc + R2 * d) * T.rs];
+      for (int h = 0; h < R1; h += PART) {
+        float2 x[PART];
 #pragma unroll
-      for (int d = 0; d < R1; ++d) {
-        const int k = jc + R2 * d;
-        float il, im, sm;
-        const int m = mode_bin(k, il, im, sm);
-        float2 p = m >= 0 ? cscale(v[d], sm) : make_float2(0.f, 0.f);
-        fp.ph[colo + (long long)k * T.rs] = p;
-        eK.add(wk * (p.x * p.x + p.y * p.y) * im);
-        float2 xx = m >= 0 ? x[d] : make_float2(0.f, 0.f);
-        eP.add(wk * (xx.x * xx.x + xx.y * xx.y) * il);
-        v[d] = xx;
+        for (int q = 0; q < PART; ++q) x[q] = dsel(fp, cur)[colo + (long long)(jc + R2 * (h + q)) * T.rs];
+#pragma unroll
+        for (int q = 0; q < PART; ++q) {
+          const int d = h + q, k = jc + R2 * d;
+          float il, im, sm;
+          const int m = mode_bin(k, il, im, sm);
+          float2 p = m >= 0 ? cscale(v[d], sm) : make_float2(0.f, 0.f);
+          __stcs(fp.ph + colo + (long long)k * T.rs, p);
+          eK.add(wk * (p.x * p.x + p.y * p.y) * im);
+          float2 xx = m >= 0 ? x[q] : make_float2(0.f, 0.f);
+          eP.add(wk * (xx.x * xx.x + xx.y * xx.y) * il);
+          v[d] = xx;
+        }
       }
     }
     fft2<N, R2, R1, INV, MAP_COL, F, TwSquare<N>::value>(v, s_ex, s_tw, t);
@@ -260,21 +282,18 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
     const float eps = (float)ds->eps;
     const float ek = first ? 0.5f * eps : eps;
     float eG = 0.f;   // X_LEAPG: sum w |g|^2 / M of the force at the start point
-    // the column in parts: the loads of a part in flight together, at a
-    // fraction of the registers of a whole column
-    constexpr int HALF = R1 / BPS_XLEAP_CHUNKS > 0 ? R1 / BPS_XLEAP_CHUNKS : 1;
     if (act) {
 #pragma unroll
-      for (int h = 0; h < R1; h += HALF) {
-      float2 x[HALF], p[HALF];
+      for (int h = 0; h < R1; h += PART) {
+      float2 x[PART], p[PART];
 #pragma unroll
-      for (int q = 0; q < HALF; ++q) {
+      for (int q = 0; q < PART; ++q) {
         const long long idx = colo + (long long)(jc + R2 * (h + q)) * T.rs;
         x[q] = src[idx];
         p[q] = fp.ph[idx];
       }
 #pragma unroll
-      for (int q = 0; q < HALF; ++q) {
+      for (int q = 0; q < PART; ++q) {
         const int d = h + q;
         const int k = jc + R2 * d;
         float il, im, sm;
@@ -320,27 +339,30 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
     const float ek = 0.5f * eps;
     TwoSumAcc eK, eP;
     float eG = 0.f;   // sum w |g|^2 / M of the last force (the Delta H identity of k_move_end)
-    float2 x[R1], p[R1];
     if (act) {
 #pragma unroll
-      for (int d = 0; d < R1; ++d) {
-        const long long idx = colo + (long long)(jc + R2 * d) * T.rs;
-        x[d] = src[idx];
-        p[d] = fp.ph[idx];
-      }
+      for (int h = 0; h < R1; h += PART) {
+        float2 x[PART], p[PART];
 #pragma unroll
-      for (int d = 0; d < R1; ++d) {
-        const int k = jc + R2 * d;
-        float il, im, sm;
-        const int m = mode_bin(k, il, im, sm);
-        if (m >= 0) {
-          float2 xx = x[d], pp = p[d];
-          const float gx = fmaf(xx.x, il, v[d].x), gy = fmaf(xx.y, il, v[d].y);
-          eG += wk * (gx * gx + gy * gy) * im;
-          pp.x = fmaf(-ek, gx, pp.x);
-          pp.y = fmaf(-ek, gy, pp.y);
-          eK.add(wk * (pp.x * pp.x + pp.y * pp.y) * im);
-          eP.add(wk * (xx.x * xx.x + xx.y * xx.y) * il);
+        for (int q = 0; q < PART; ++q) {
+          const long long idx = colo + (long long)(jc + R2 * (h + q)) * T.rs;
+          x[q] = src[idx];
+          p[q] = fp.ph[idx];
+        }
+#pragma unroll
+        for (int q = 0; q < PART; ++q) {
+          const int d = h + q, k = jc + R2 * d;
+          float il, im, sm;
+          const int m = mode_bin(k, il, im, sm);
+          if (m >= 0) {
+            float2 xx = x[q], pp = p[q];
+            const float gx = fmaf(xx.x, il, v[d].x), gy = fmaf(xx.y, il, v[d].y);
+            eG += wk * (gx * gx + gy * gy) * im;
+            pp.x = fmaf(-ek, gx, pp.x);
+            pp.y = fmaf(-ek, gy, pp.y);
+            eK.add(wk * (pp.x * pp.x + pp.y * pp.y) * im);
+            eP.add(wk * (xx.x * xx.x + xx.y * xx.y) * il);
+          }
         }
       }
     }
@@ -359,20 +381,23 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   if constexpr (MODE == X_GRAD) {
     TwoSumAcc eP;
     if (act) {
-      float2 x[R1];
 #pragma unroll
-      for (int d = 0; d < R1; ++d) x[d] = dsel(fp, cur)[colo + (long long)(jc + R2 * d) * T.rs];
+      for (int h = 0; h < R1; h += PART) {
+        float2 x[PART];
 #pragma unroll
-      for (int d = 0; d < R1; ++d) {
-        const int k = jc + R2 * d;
-        float il, im, sm;
-        const int m = mode_bin(k, il, im, sm);
-        float2 g = make_float2(0.f, 0.f);
-        if (m >= 0) {
-          g = make_float2(fmaf(x[d].x, il, v[d].x), fmaf(x[d].y, il, v[d].y));
-          eP.add(wk * (x[d].x * x[d].x + x[d].y * x[d].y) * il);
+        for (int q = 0; q < PART; ++q) x[q] = dsel(fp, cur)[colo + (long long)(jc + R2 * (h + q)) * T.rs];
+#pragma unroll
+        for (int q = 0; q < PART; ++q) {
+          const int d = h + q, k = jc + R2 * d;
+          float il, im, sm;
+          const int m = mode_bin(k, il, im, sm);
+          float2 g = make_float2(0.f, 0.f);
+          if (m >= 0) {
+            g = make_float2(fmaf(x[q].x, il, v[d].x), fmaf(x[q].y, il, v[d].y));
+            eP.add(wk * (x[q].x * x[q].x + x[q].y * x[q].y) * il);
+          }
+          xa.dst[dst_idx(k)] = g;
         }
-        xa.dst[dst_idx(k)] = g;
       }
     }
     double sP = block_sum2<NT>(eP, reinterpret_cast<float*>(s_red));
@@ -964,6 +989,13 @@ struct ZSmem {
   static constexpr size_t OFF_RED = OFF_TW + (size_t)N * sizeof(float2);
   static constexpr size_t OFF_BAR = OFF_RED + 32 * sizeof(double);
   static constexpr size_t BYTES = OFF_BAR + sizeof(uint64_t);
+  // Z_SUMS: the threads' sums of each quantity behind the rest, rows of NTZ floats
+  // padded so that four rows fall on different banks
+  static constexpr int ACCP = LP * C::RMAX + 8;
+  static constexpr size_t OFF_ACC = (BYTES + 15) / 16 * 16;
+  __host__ __device__ static constexpr size_t bytes(int n_sub) {
+    return MODE == Z_SUMS ? OFF_ACC + 3 * (size_t)n_sub * ACCP * sizeof(float) : BYTES;
+  }
   static_assert(BUF >= (size_t)LINES * C::ZP * sizeof(float2), "staging does not fit");
   static_assert(BUF >= (size_t)LINES * N * sizeof(float), "staging does not fit");
 };
@@ -1143,55 +1175,90 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
       return;
     }
     if constexpr (MODE == Z_SUMS) {
+      // delta of the tile through shared memory (the exchange buffer, [LINES][N]), so
+      // that sixteen lanes share a line's support in 16-byte loads of R and 8-byte
+      // loads of the counts, three subsamples' in flight, with the transform's
+      // registers free again.  A thread's FP32 sums of its terms (at most 32 for a dense
+      // survey) go to shared memory per quantity, and eight lanes add each quantity's
+      // as compensated pairs: one reduction per tile instead of five shuffle steps per
+      // quantity and warp, which were most of this pass's instructions (111 registers,
+      // 22% of the warp slots, 84 us at 256^3 with six subsamples, 35 us at 128^3 with
+      // fifteen; now 42 and 22 us).
       const long long nv = (long long)N * N * N;
       const int nsub = ds->nsub;
-      const int loa = f < LP ? s_lo[2 * f] : 0, hia = f < LP ? s_hi[2 * f] : 0;
-      const int lob = f < LP ? s_lo[2 * f + 1] : 0, hib = f < LP ? s_hi[2 * f + 1] : 0;
-      // per-warp sums of all 3 nsub quantities as compensated FP32 pairs, then one
-      // pass over the warps (the same additions, in the same order, as one block
-      // sum per quantity)
-      constexpr int NW = (NTZ + 31) / 32;
-      __shared__ float s_ws[NW][3 * MAXS][2];   // compensated pairs
-      const int lane = t & 31, w = t >> 5;
-      for (int l = 0; l < nsub; ++l) {
-        float s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        if (f < LP) {
-          const uint16_t* cn = sd.cnt + l * nv;
-          const float* rr = sd.R + l * nv;
+      float* s_d = reinterpret_cast<float*>(s_buf);
+      float* s_acc = reinterpret_cast<float*>(smem + L::OFF_ACC);   // [3 nsub][ACCP]
+      constexpr int ACCP = L::ACCP;
+      if (f < LP) {
 #pragma unroll
-          for (int d = 0; d < R2; ++d) {
-            const int n = c + R1 * d;
-            const bool ina = n >= loa && n < hia, inb = n >= lob && n < hib;
-            const float da = v[d].x * fp.inv_nv, db = v[d].y * fp.inv_nv;
-            const float ra = ina ? rr[la + n] : 0.f, rb = inb ? rr[lb + n] : 0.f;
-            const float na = ina ? (float)cn[la + n] : 0.f, nb = inb ? (float)cn[lb + n] : 0.f;
-            s1 += na * da + nb * db;
-            s2 += ra * da + rb * db;
-            s3 += ra * da * da + rb * db * db;
-          }
-        }
-        float c1 = 0.f, c2 = 0.f, c3 = 0.f;
-        warp_sum2<NTZ>(s1, c1);
-        warp_sum2<NTZ>(s2, c2);
-        warp_sum2<NTZ>(s3, c3);
-        if (lane == 0) {
-          s_ws[w][3 * l + 0][0] = s1;
-          s_ws[w][3 * l + 0][1] = c1;
-          s_ws[w][3 * l + 1][0] = s2;
-          s_ws[w][3 * l + 1][1] = c2;
-          s_ws[w][3 * l + 2][0] = s3;
-          s_ws[w][3 * l + 2][1] = c3;
+        for (int d = 0; d < R2; ++d) {
+          const int n = c + R1 * d;
+          s_d[(2 * f) * N + n] = v[d].x * fp.inv_nv;
+          s_d[(2 * f + 1) * N + n] = v[d].y * fp.inv_nv;
         }
       }
       __syncthreads();
-      for (int q = t; q < 3 * nsub; q += NTZ) {
-        TwoSumAcc r;
+      constexpr int G = 3;                        // subsamples at a time
+      constexpr int LPL = N / 4 < 16 ? N / 4 : 16;   // lanes per line
+      constexpr bool SHORT = N <= 64;             // one float4 group per lane covers a line
+      constexpr int LPR = NTZ / LPL;              // lines per round
+      static_assert(!SHORT || LINES % LPR == 0, "lines in whole rounds");
+      for (int l0 = 0; l0 < nsub; l0 += G) {
+        float s1[G] = {}, s2[G] = {}, s3[G] = {};
+        // the group of four voxels z of line ln, if inside the support
+        auto add = [&](int ln, int z) {
+          float4 r[G];
+          ushort4 n[G];
+          const bool here = z >= s_lo[ln] && z < s_hi[ln];
 #pragma unroll
-        for (int i = 0; i < NW; ++i) {
-          r.add(s_ws[i][q][0]);
-          r.add(s_ws[i][q][1]);
+          for (int g = 0; g < G; ++g) {
+            const bool in = here && l0 + g < nsub;
+            const long long i = (l0 + g) * nv + (L0 + ln) * N + z;
+            r[g] = in ? __ldg(reinterpret_cast<const float4*>(sd.R + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            n[g] = in ? __ldg(reinterpret_cast<const ushort4*>(sd.cnt + i)) : make_ushort4(0, 0, 0, 0);
+          }
+          const float4 d4 = *reinterpret_cast<const float4*>(s_d + ln * N + z);
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            const float rx = r[g].x * d4.x, ry = r[g].y * d4.y, rz = r[g].z * d4.z, rw = r[g].w * d4.w;
+            s1[g] += ((float)n[g].x * d4.x + (float)n[g].y * d4.y) + ((float)n[g].z * d4.z + (float)n[g].w * d4.w);
+            s2[g] += (rx + ry) + (rz + rw);
+            s3[g] += (rx * d4.x + ry * d4.y) + (rz * d4.z + rw * d4.w);
+          }
+        };
+        if constexpr (SHORT) {
+#pragma unroll
+          for (int i = 0; i < LINES / LPR; ++i) add(t / LPL + i * LPR, 4 * (t % LPL));
+        } else {
+          for (int ln = t / LPL; ln < LINES; ln += LPR) {
+            for (int z = s_lo[ln] + 4 * (t % LPL); z < s_hi[ln]; z += 4 * LPL) add(ln, z);
+          }
         }
-        fp.part[za.region + q * fp.part_stride + blockIdx.x] = r.value();
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          if (l0 + g < nsub) {
+            float* p = s_acc + 3 * (l0 + g) * ACCP + t;
+            p[0] = s1[g];
+            p[ACCP] = s2[g];
+            p[2 * ACCP] = s3[g];
+          }
+        }
+      }
+      __syncthreads();
+      const int sub = t & 7;
+      constexpr unsigned MASK = NTZ >= 32 ? 0xffffffffu : ((1u << NTZ) - 1u);
+      for (int q0 = 0; q0 < 3 * nsub; q0 += NTZ / 8) {
+        const int q = q0 + (t >> 3);
+        TwoSumAcc r;
+        if (q < 3 * nsub)
+          for (int i = sub; i < NTZ; i += 8) r.add(s_acc[q * ACCP + i]);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+          const float os = __shfl_down_sync(MASK, r.s, o, 8), oc = __shfl_down_sync(MASK, r.c, o, 8);
+          r.add(os);
+          r.c = __fadd_rn(r.c, oc);
+        }
+        if (sub == 0 && q < 3 * nsub) fp.part[za.region + q * fp.part_stride + blockIdx.x] = r.value();
       }
       return;
     }
@@ -1427,32 +1494,50 @@ __global__ void __launch_bounds__(256) k_rebuild(Fields fp0, long long nv, int r
   __syncthreads();
   float acc = 0.f, comp = 0.f;   // FP32 with Kahan compensation per thread; FP64 across the block
   const SurveyData sd = survey(fp);
-  // a and c of the four voxels of float4 group i
+  // a and c of the four voxels of float4 group i, the data of three subsamples in flight
   auto group = [&](long long i) -> float {
+    constexpr int G = 3;
     float4 A = make_float4(0.f, 0.f, 0.f, 0.f), Cc = A;
-    for (int l = 0; l < nsub; ++l) {
-      const float4 r = reinterpret_cast<const float4*>(sd.R + l * nv)[i];
-      const ushort4 n = reinterpret_cast<const ushort4*>(sd.cnt + l * nv)[i];
-      const float ka = s_a[l], kb = s_b[l], kbn = s_bn[l];
-      A.x = fmaf(ka, r.x, A.x); A.y = fmaf(ka, r.y, A.y); A.z = fmaf(ka, r.z, A.z); A.w = fmaf(ka, r.w, A.w);
-      Cc.x += kb * (float)n.x - kbn * r.x;
-      Cc.y += kb * (float)n.y - kbn * r.y;
-      Cc.z += kb * (float)n.z - kbn * r.z;
-      Cc.w += kb * (float)n.w - kbn * r.w;
+    for (int l0 = 0; l0 < nsub; l0 += G) {
+      float4 r[G];
+      ushort4 n[G];
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const bool in = l0 + g < nsub;
+        r[g] = in ? reinterpret_cast<const float4*>(sd.R + (l0 + g) * nv)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        n[g] = in ? reinterpret_cast<const ushort4*>(sd.cnt + (l0 + g) * nv)[i] : make_ushort4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        if (l0 + g < nsub) {
+          const float ka = s_a[l0 + g], kb = s_b[l0 + g], kbn = s_bn[l0 + g];
+          A.x = fmaf(ka, r[g].x, A.x); A.y = fmaf(ka, r[g].y, A.y); A.z = fmaf(ka, r[g].z, A.z); A.w = fmaf(ka, r[g].w, A.w);
+          Cc.x += kb * (float)n[g].x - kbn * r[g].x;
+          Cc.y += kb * (float)n[g].y - kbn * r[g].y;
+          Cc.z += kb * (float)n[g].z - kbn * r[g].z;
+          Cc.w += kb * (float)n[g].w - kbn * r[g].w;
+        }
+      }
     }
     reinterpret_cast<float4*>(fp.a)[i] = A;
     reinterpret_cast<float4*>(fp.c)[i] = Cc;
     return (A.x + A.y) + (A.z + A.w);
   };
   if (sd.span) {
-    // one warp per z line, its lanes over the line's support (multiples of 4 voxels)
+    // half a warp per z line, its lanes over the line's support (multiples of 4 voxels,
+    // mostly less than 64), the next line's support on its way: a chain of latencies,
+    // 39 us at 256^3 with six subsamples and 73 us for 32 chains of 96^3 with a warp per
+    // line and one load at a time, now 28 and 49 us
     const int n_grid = fp.grid_n;
     const int lines = n_grid * n_grid, gpl = n_grid / 4;   // float4 groups per line
-    const int lane = threadIdx.x & 31;
-    for (int line = blockIdx.x * 8 + (threadIdx.x >> 5); line < lines; line += gridDim.x * 8) {
-      const int2 sp = sd.span[line];
+    const int lane = threadIdx.x & 15, step = gridDim.x * 16;
+    int line = blockIdx.x * 16 + (threadIdx.x >> 4);
+    int2 next = line < lines ? sd.span[line] : make_int2(0, 0);
+    for (; line < lines; line += step) {
+      const int2 sp = next;
+      if (line + step < lines) next = sd.span[line + step];
       const int g0 = (n_grid - sp.x) / 4, g1 = sp.y / 4;
-      for (int g = g0 + lane; g < g1; g += 32) kahan_add(acc, comp, group((long long)line * gpl + g));
+      for (int g = g0 + lane; g < g1; g += 16) kahan_add(acc, comp, group((long long)line * gpl + g));
     }
   } else {
     const long long n4 = nv / 4;
@@ -1695,12 +1780,13 @@ struct Launch {
   }
   template <int M, int LP = C::LP>
   static void z(const Fields& fp, const ZArgs& za, int nch, cudaStream_t s) {
-    launch_dep(k_zpass<N, M, LP>, dim3(N * N / (2 * LP), nch), dim3(LP * C::RMAX), ZSmem<N, M, LP>::BYTES, s, fp, za);
+    launch_dep(k_zpass<N, M, LP>, dim3(N * N / (2 * LP), nch), dim3(LP * C::RMAX),
+               ZSmem<N, M, LP>::bytes(fp.n_sub), s, fp, za);
   }
   template <int M, int LP = C::LP>
   static void zattr() {
     cudaFuncSetAttribute(k_zpass<N, M, LP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)ZSmem<N, M, LP>::BYTES);
+                         (int)ZSmem<N, M, LP>::bytes(MAXS));
   }
   static void attrs() {
     zattr<Z_GRAD>(); zattr<Z_NOISE>(); zattr<Z_R2C>(); zattr<Z_C2R>(); zattr<Z_SUMS>();
