@@ -309,7 +309,6 @@ ScalarArgs scalars(bps_ctx* c) {
   a.n_mass = c->n_mass;
   a.inv_nv = 1.0 / (double)c->nv;
   a.alpha = c->cfg.alpha;
-  a.eps_max = c->cfg.eps_max;
   a.jeps_max = c->cfg.jump_eps_max;
   a.fixed_bias = c->cfg.fixed_bias_index;
   return a;
@@ -487,8 +486,7 @@ bps_status hmc_move(bps_ctx* ctx, bool advance) {
   const PassTable& P = ctx->pt;
   const int L = ctx->cfg.n_leapfrog, B = ctx->batch;
   if (ctx->mnet) launch_mass_net(sa, ctx->mnet, B, s);
-  launch_move_begin(sa, B, s);
-  P.z_noise(f, B, s);
+  P.z_noise(f, ctx->cfg.eps_max, B, s);
   P.y_fwd(f, BUF_PH, B, s);
   P.x_init(f, region_offset(ctx, RG_INIT), B, s);
   bps_status sf = force_stage(ctx, f, region_offset(ctx, RG_LIK0), false, s);
@@ -505,7 +503,7 @@ bps_status hmc_move(bps_ctx* ctx, bool advance) {
   P.x_final(f, region_offset(ctx, RG_FINAL), B, s);
   launch_move_end(sa, region_offset(ctx, RG_INIT), region_offset(ctx, RG_LIK0), region_offset(ctx, RG_FINAL),
                   region_offset(ctx, RG_LIK1), P.x_tiles, lik_tiles(ctx), advance ? 1 : 0, B, s);
-  LAUNCHED(ctx, 6 + L + (ctx->mnet ? 1 : 0));
+  LAUNCHED(ctx, 5 + L + (ctx->mnet ? 1 : 0));
   return BPS_OK;
 }
 
@@ -2234,13 +2232,12 @@ bps_status bps_gradient(bps_ctx* ctx, float* grad_dev, double* energies) {
   Fields f = fields_at(ctx, 0);
   ScalarArgs sa = scalars_at(ctx, 0);
   cudaStream_t s = ctx->stream;
-  launch_move_begin(sa, 1, s);   // per-bin tables of the current P and abar
-  ctx->pt.x_inv(f, -1, ctx->W, 1, s);
+  ctx->pt.x_inv_tables(f, ctx->cfg.eps_max, s);   // with the per-bin tables of the current P and abar
   bps_status sf = force_stage(ctx, f, region_offset(ctx, RG_LIK0), false, s);
   if (sf != BPS_OK) return sf;
   const bool direct = aligned8(grad_dev);
   ctx->pt.x_grad(f, direct ? reinterpret_cast<float2*>(grad_dev) : ctx->W, direct, region_offset(ctx, RG_GRAD), s);
-  LAUNCHED(ctx, 3);
+  LAUNCHED(ctx, 2);
   if (!direct) {
     st = copy_spec_out(ctx, ctx->W, grad_dev);
     if (st != BPS_OK) return st;

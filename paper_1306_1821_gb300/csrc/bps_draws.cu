@@ -37,39 +37,6 @@ __device__ double sum_partials(const double* p, int n, double* sh) {
 // read, and small kernels that only consume what another one finishes are that
 // one's last block.
 
-// Per-bin tables of the move and its scalars: two warps per table column (a
-// division and a square root each), one for the step size and the Metropolis draw.
-__global__ void __launch_bounds__(288) k_move_begin(ScalarArgs a0) {
-  await_previous();
-  const ScalarArgs a = chain_args(a0, blockIdx.y);
-  DevState* ds = a.ds;
-  const int t = threadIdx.x & 63, role = threadIdx.x >> 6;
-  if (role == 4) {
-    if (t == 0) {
-      P4 r = philox(0, ds->iteration, ST_HMC, 0, ds->seed);
-      ds->eps = a.eps_max * u52(r.w[0]);
-      ds->log_u = log(u52(r.w[1]));
-    }
-    return;
-  }
-  if (role < 2) {
-    // lambda_m = P_m / V_cell (Eq. dens_prior in Fourier space); M = 1/lambda + abar (Eq. Mass_matrix)
-    const bool bin = t < a.n_bins;
-    const double il = bin ? ds->vc / ds->P[t] : 0.0;
-    const double M = il + ds->abar;
-    if (role == 0) {
-      ds->inv_lambda[t] = (float)il;
-      ds->inv_M[t] = bin ? (float)(1.0 / M) : 0.f;
-    } else {
-      ds->sqrt_M[t] = bin ? (float)sqrt(M) : 0.f;
-    }
-  } else {
-    const double sc = t < a.n_mass ? ds->mass_scale[t] : 1.0;
-    if (role == 2) ds->inv_ms[t] = (float)(1.0 / sc);
-    else ds->sqrt_ms[t] = (float)sqrt(sc);
-  }
-}
-
 // H = (1/2N^3) sum w (|p|^2/M + |delta|^2/lambda) + (1/2) sum (a delta^2 - 2 c delta)
 // The eight sums of a move, one block each (on different SMs: each sum is a
 // chain of FP64 additions), into the chain state's scratch: K0, E0, L0, K1, E1,
@@ -596,9 +563,6 @@ __global__ void k_mstat(ScalarArgs a0, int region, int nblk, int final_) {
   }
 }
 
-void launch_move_begin(const ScalarArgs& a, int nch, cudaStream_t s) {
-  launch_dep(k_move_begin, dim3(1, nch), dim3(288), 0, s, a);
-}
 void launch_move_end(const ScalarArgs& a, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz, int advance,
                      int nch, cudaStream_t s) {
   launch_dep(k_move_end, dim3(8, nch), dim3(256), 0, s, a, r_init, r_lik0, r_final, r_lik1, nx, nz, advance);

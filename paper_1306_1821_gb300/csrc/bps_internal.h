@@ -63,7 +63,10 @@ struct PassTable {
   void (*y_fwd)(const Fields&, int buf, int nch, cudaStream_t);
   void (*y_inv)(const Fields&, int buf, int nch, cudaStream_t);
   void (*z_grad)(const Fields&, int region, int nch, cudaStream_t);
-  void (*z_noise)(const Fields&, int nch, cudaStream_t);
+  // the momentum normals' z transform, and the move tables with this step size bound
+  void (*z_noise)(const Fields&, double eps_max, int nch, cudaStream_t);
+  // one chain: W = IFFT_x(current state), and the move tables
+  void (*x_inv_tables)(const Fields&, double eps_max, cudaStream_t);
   void (*z_r2c)(const Fields&, const float* rin, float2* dst, cudaStream_t);   // one chain
   void (*z_c2r)(const Fields&, const float2* src, float* rout, cudaStream_t);  // one chain
   // one chain: delta = C2R_z(W) added to the running sums mom[0..N^3) (delta) and mom[N^3..) (delta^2)
@@ -126,10 +129,9 @@ struct ScalarArgs {
   int stride;
   long long cstride;
   int n_bins, max_sub, n_mass;
-  double inv_nv, alpha, eps_max, jeps_max;
+  double inv_nv, alpha, jeps_max;
   int fixed_bias;
 };
-void launch_move_begin(const ScalarArgs& a, int nch, cudaStream_t s);
 // advance = 1: and move the iteration counter on
 void launch_move_end(const ScalarArgs& a, int r_init, int r_lik0, int r_final, int r_lik1, int nx, int nz, int advance,
                      int nch, cudaStream_t s);

@@ -47,6 +47,7 @@ struct XArgs {
   int first;
   int region;    // offset (doubles) of this launch's partial sums in Fields::part
   const float* amp = nullptr;   // X_AMP: amplitude of every |n|^2
+  double eps_max = -1.0;        // X_INV: unless negative, one more block per chain makes the move tables
   int unpadded = 0;             // X_GRAD, X_FWD: dst is a caller's half spectrum [N][N][N/2+1]
 };
 
@@ -63,6 +64,7 @@ struct ZArgs {
   // Z_NOISE with a stage: the normals of stream (seed, 0, stage, 0) into dst
   // instead of the move's momentum into the momentum spectrum
   uint64_t stage = 0;
+  double eps_max = -1.0;  // Z_NOISE: unless negative, one more block per chain makes the move tables
 };
 
 // ------------------------------------------------------------------ x pass helpers
@@ -148,6 +150,12 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   DevState* ds = fp.ds;
   load_twiddles<N>(s_tw, fp.tw, t, NT);
   await_previous();
+  if constexpr (MODE == X_INV) {
+    if (blockIdx.x == C::TILES) {
+      move_tables(fp, xa.eps_max, t, NT);
+      return;
+    }
+  }
   if constexpr (MODE == X_SCALE) {
     if (!ds->jaccepted) return;   // uniform across the grid
   }
@@ -1018,10 +1026,16 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
   if constexpr (MODE == Z_GRAD) {
     if (ds->jreuse) return;       // force stage reused by the jump (uniform)
   }
+  if constexpr (MODE == Z_NOISE) {
+    if (blockIdx.x == N * N / LINES) {
+      move_tables(fp, za.eps_max, t, NTZ);
+      return;
+    }
+  }
   // Lines in decreasing x: the y passes visit the x planes upwards, so the planes
   // the z pass reads first are the ones the inverse y pass wrote last (still in
   // L2), and the forward y pass starts on the planes the z pass wrote last.
-  const long long L0 = (long long)(gridDim.x - 1 - blockIdx.x) * LINES;
+  const long long L0 = (long long)(N * N / LINES - 1 - (int)blockIdx.x) * LINES;
   constexpr bool STAGED = MODE != Z_NOISE;
   // Z_GRAD, Z_SUMS: support [lo, hi) of R on each line of the tile (whole lines
   // without support information).  Outside it R = 0, the counts are 0 and
@@ -1772,7 +1786,7 @@ struct Launch {
   using C = Cfg<N>;
   template <int M>
   static void x(const Fields& fp, const XArgs& xa, int nch, cudaStream_t s) {
-    launch_dep(k_xpass<N, M>, dim3(C::TILES, nch), dim3(C::NT), 0, s, fp, xa);
+    launch_dep(k_xpass<N, M>, dim3(C::TILES + (M == X_INV && xa.eps_max >= 0.0), nch), dim3(C::NT), 0, s, fp, xa);
   }
   template <int D>
   static void y(const Fields& fp, int buf, int nch, cudaStream_t s) {
@@ -1780,7 +1794,7 @@ struct Launch {
   }
   template <int M, int LP = C::LP>
   static void z(const Fields& fp, const ZArgs& za, int nch, cudaStream_t s) {
-    launch_dep(k_zpass<N, M, LP>, dim3(N * N / (2 * LP), nch), dim3(LP * C::RMAX),
+    launch_dep(k_zpass<N, M, LP>, dim3(N * N / (2 * LP) + (za.eps_max >= 0.0), nch), dim3(LP * C::RMAX),
                ZSmem<N, M, LP>::bytes(fp.n_sub), s, fp, za);
   }
   template <int M, int LP = C::LP>
@@ -1811,8 +1825,8 @@ static PassTable make_table() {
   T.x_final = [](const Fields& f, int region, int n, cudaStream_t s) { L::template x<X_FINAL>(f, XArgs{-1, nullptr, 0, region}, n, s); };
   T.x_inv = [](const Fields& f, int src, float2* dst, int n, cudaStream_t s) { L::template x<X_INV>(f, XArgs{src, dst, 0, -1}, n, s); };
   T.x_fwd = [](const Fields& f, int src, float2* dst, int n, cudaStream_t s) { L::template x<X_FWD>(f, XArgs{src, dst, 0, -1}, n, s); };
-  T.x_grad = [](const Fields& f, float2* dst, bool unpadded, int region, cudaStream_t s) { L::template x<X_GRAD>(f, XArgs{-1, dst, 0, region, nullptr, unpadded}, 1, s); };
-  T.x_out = [](const Fields& f, float2* dst, cudaStream_t s) { L::template x<X_FWD>(f, XArgs{BUF_W, dst, 0, -1, nullptr, 1}, 1, s); };
+  T.x_grad = [](const Fields& f, float2* dst, bool unpadded, int region, cudaStream_t s) { L::template x<X_GRAD>(f, XArgs{-1, dst, 0, region, nullptr, -1.0, unpadded}, 1, s); };
+  T.x_out = [](const Fields& f, float2* dst, cudaStream_t s) { L::template x<X_FWD>(f, XArgs{BUF_W, dst, 0, -1, nullptr, -1.0, 1}, 1, s); };
   T.x_jinv = [](const Fields& f, int n, cudaStream_t s) { L::template x<X_JINV>(f, XArgs{-1, nullptr, 0, -1}, n, s); };
   T.x_jgrad = [](const Fields& f, int region, int n, cudaStream_t s) { L::template x<X_JGRAD>(f, XArgs{-1, nullptr, 0, region}, n, s); };
   T.x_scale = [](const Fields& f, int n, cudaStream_t s) { L::template x<X_SCALE>(f, XArgs{-1, nullptr, 0, -1}, n, s); };
@@ -1828,7 +1842,8 @@ static PassTable make_table() {
   T.z_grad_lp[1] = [](const Fields& f, int region, int n, cudaStream_t s) { L::template z<Z_GRAD, 8>(f, ZArgs{nullptr, nullptr, nullptr, nullptr, region, 0}, n, s); };
   T.z_grad_lp[2] = [](const Fields& f, int region, int n, cudaStream_t s) { L::template z<Z_GRAD, 16>(f, ZArgs{nullptr, nullptr, nullptr, nullptr, region, 0}, n, s); };
   for (int i = 0; i < 3; ++i) T.z_lp_tiles[i] = N * N / (2 * (4 << i));
-  T.z_noise = [](const Fields& f, int n, cudaStream_t s) { L::template z<Z_NOISE>(f, ZArgs{nullptr, nullptr, nullptr, nullptr, -1, 0}, n, s); };
+  T.z_noise = [](const Fields& f, double eps_max, int n, cudaStream_t s) { L::template z<Z_NOISE>(f, ZArgs{nullptr, nullptr, nullptr, nullptr, -1, 0, nullptr, 0, eps_max}, n, s); };
+  T.x_inv_tables = [](const Fields& f, double eps_max, cudaStream_t s) { L::template x<X_INV>(f, XArgs{-1, nullptr, 0, -1, nullptr, eps_max}, 1, s); };
   T.x_amp = [](const Fields& f, const float* amp, cudaStream_t s) { L::template x<X_AMP>(f, XArgs{-1, nullptr, 0, -1, amp}, 1, s); };
   T.z_mock = [](const Fields& f, uint64_t seed, uint64_t stage, float2* dst, cudaStream_t s) { L::template z<Z_NOISE>(f, ZArgs{nullptr, dst, nullptr, nullptr, -1, seed, nullptr, stage}, 1, s); };
   T.z_r2c = [](const Fields& f, const float* rin, float2* dst, cudaStream_t s) { L::template z<Z_R2C>(f, ZArgs{nullptr, dst, rin, nullptr, -1, 0}, 1, s); };

@@ -87,6 +87,39 @@ __host__ __device__ __forceinline__ Fields at_chain(Fields f, int ch) {
   return f;
 }
 
+// The scalars and per-bin tables of a move, by one block of nt threads: the step
+// size and the Metropolis draw, lambda_m = P_m / V_cell (Eq. dens_prior in Fourier
+// space) and M = 1/lambda + abar (Eq. Mass_matrix) with their roots and inverses.
+// They are FP64 divisions and square roots, most of a microsecond each, so each
+// thread takes one and they run as one more block of a kernel that does not need
+// them: the z pass that draws the momentum normals, or the inverse x pass of a
+// force evaluation (a kernel of their own: 4.2 us in the chain of launches).
+__device__ __forceinline__ void move_tables(const Fields& fp, double eps_max, int t, int nt) {
+  DevState* ds = fp.ds;
+  for (int q = t; q <= 4 * MAXB; q += nt) {
+    const int m = q % MAXB, role = q / MAXB;
+    if (role == 4) {
+      const P4 r = philox(0, ds->iteration, ST_HMC, 0, ds->seed);
+      ds->eps = eps_max * u52(r.w[0]);
+      ds->log_u = log(u52(r.w[1]));
+    } else if (role < 2) {
+      const bool bin = m < fp.n_bins;
+      const double il = bin ? ds->vc / ds->P[m] : 0.0;
+      const double M = il + ds->abar;
+      if (role == 0) {
+        ds->inv_lambda[m] = (float)il;
+        ds->inv_M[m] = bin ? (float)(1.0 / M) : 0.f;
+      } else {
+        ds->sqrt_M[m] = bin ? (float)sqrt(M) : 0.f;
+      }
+    } else {
+      const double sc = m < fp.n_mass ? ds->mass_scale[m] : 1.0;
+      if (role == 2) ds->inv_ms[m] = (float)(1.0 / sc);
+      else ds->sqrt_ms[m] = (float)sqrt(sc);
+    }
+  }
+}
+
 enum { MAP_COL = 0, MAP_ROW = 1 };
 
 template <int MAP, int A, int B, int F>
