@@ -208,11 +208,12 @@ __device__ __forceinline__ int gauss_count(float r, float d, double b, double nb
 // read once.  FP64 issue bounds any FP64 work here: 13.8 ms at 256^3 with six
 // subsamples with every voxel searched in FP64, 1.72 ms with lambda in FP64 and
 // the search in FP32 at the observed voxels only (FP64 pipe 77% busy), and
-// 0.55 ms with lambda in FP32 pairs as well: ALU and FMA pipes 35% and 29% busy,
-// the rest loads.  Four voxels per thread hold 124 registers and two blocks per
-// SM (0.92 ms); one response in flight per thread instead of four takes 0.70 ms.
+// 0.55 ms with lambda in FP32 pairs as well, 0.42 ms with the registers cut from 64 to
+// 36 for seven blocks per SM instead of four (0.45 ms with six or eight): latency.
+// Four voxels per thread hold 124 registers and two blocks per SM (0.92 ms); one
+// response in flight per thread instead of four takes 0.70 ms.
 template <int NOISE>
-__global__ void __launch_bounds__(256, 4) k_mock_counts(const float* __restrict__ delta, const float* __restrict__ R,
+__global__ void __launch_bounds__(256, 7) k_mock_counts(const float* __restrict__ delta, const float* __restrict__ R,
                                                         long long nv, int nsub, MockSub sub, uint64_t seed,
                                                         int32_t* __restrict__ out) {
   constexpr int G = 4;   // responses in flight per thread: most voxels only pass through
