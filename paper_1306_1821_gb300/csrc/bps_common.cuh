@@ -183,7 +183,12 @@ struct Cfg {
   static constexpr int RMAX = R1 > R2 ? R1 : R2;
   static constexpr int H = N / 2;                      // Nyquist index
   static constexpr int ZP = ((H + 1) + 1) / 2 * 2;     // padded row length (complex)
-  static constexpr int F = H < 16 ? H : 16;            // tile columns
+  // Tile columns: 16 (rows of 128 bytes).  At 128^3 that makes 520 tiles of 256 threads
+  // for about as many places on the GPU, and a second, nearly empty wave; 8 columns
+  // make 1040 tiles of 128 threads: 128^3 with fifteen subsamples 728 -> 707 us per Gibbs
+  // iteration.  256^3 has 2064 tiles, the smaller grids one wave.
+  static constexpr int F = H < 16 ? H : N == 128 ? 8 : 16;
+  static constexpr int PER_256 = N == 128 ? 2 : 1;     // tiles of this grid per 256 threads, for launch bounds
   static constexpr int NT = F * RMAX < 32 ? 32 : F * RMAX;  // threads per strided tile
   static constexpr int LP = BPS_ZPAIRS;                // line pairs per contiguous-axis tile
   static constexpr int NTZ = LP * RMAX;                // threads per contiguous-axis tile

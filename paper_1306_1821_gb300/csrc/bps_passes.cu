@@ -124,10 +124,10 @@ template <int N, int MODE>
 __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG || MODE == X_AMP ||
                                                       ((MODE == X_INIT || MODE == X_FINAL || MODE == X_GRAD) &&
                                                        XParts<N>::value)
-                                                  ? BPS_XLEAP_MIN_BLOCKS
-                                              : MODE == X_JINV  ? BPS_XJINV_MIN_BLOCKS
-                                              : MODE == X_JGRAD ? BPS_XJGRAD_MIN_BLOCKS
-                                                                : BPS_XPASS_MIN_BLOCKS)
+                                                  ? Cfg<N>::PER_256 * BPS_XLEAP_MIN_BLOCKS
+                                              : MODE == X_JINV  ? Cfg<N>::PER_256 * BPS_XJINV_MIN_BLOCKS
+                                              : MODE == X_JGRAD ? Cfg<N>::PER_256 * BPS_XJGRAD_MIN_BLOCKS
+                                                                : Cfg<N>::PER_256 * BPS_XPASS_MIN_BLOCKS)
     k_xpass(Fields fp0, XArgs xa) {
   const Fields fp = at_chain(fp0, blockIdx.y);
   using C = Cfg<N>;
@@ -619,7 +619,7 @@ struct XTma {
   using C = Cfg<N>;
   static constexpr int TILE = N * C::F;                    // complex elements of one tile
   static constexpr size_t SMEM = (1 + SD + SP) * (size_t)TILE * sizeof(float2);
-  static constexpr int MIN_BLOCKS = SD + SP == 2 ? 2 : 3;
+  static constexpr int MIN_BLOCKS = C::PER_256 * (SD + SP == 2 ? 2 : 3);
 };
 
 template <int N, int SD, int SP>
@@ -774,7 +774,7 @@ struct XRing {
 };
 
 template <int N, bool TMA>
-__global__ void __launch_bounds__(Cfg<N>::NT, BPS_XLEAP_MIN_BLOCKS)
+__global__ void __launch_bounds__(Cfg<N>::NT, Cfg<N>::PER_256 * BPS_XLEAP_MIN_BLOCKS)
     k_xleap_ring(Fields fp0, XArgs xa, const __grid_constant__ XMaps maps) {
   using XR = XRing<N>;
   const Fields fp = at_chain(fp0, blockIdx.y);
@@ -941,7 +941,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, BPS_XLEAP_MIN_BLOCKS)
 
 // ------------------------------------------------------------------ y pass
 template <int N, int DIR>
-__global__ void __launch_bounds__(Cfg<N>::NT, BPS_YPASS_MIN_BLOCKS) k_ypass(Fields fp0, int buf) {
+__global__ void __launch_bounds__(Cfg<N>::NT, Cfg<N>::PER_256 * BPS_YPASS_MIN_BLOCKS) k_ypass(Fields fp0, int buf) {
   const Fields fp = at_chain(fp0, blockIdx.y);
   await_previous();
   if (buf == BUF_W && fp.ds->jreuse) return;   // force stage reused by the jump (uniform)
@@ -1350,7 +1350,7 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
 // two-slot layout): the quarter loop has no block barrier, only the warp's own
 // copy-group waits and warp barriers.  Nyquist tiles read delta and p directly.
 template <int N>
-__global__ void __launch_bounds__(Cfg<N>::NT, BPS_XLEAP_MIN_BLOCKS)
+__global__ void __launch_bounds__(Cfg<N>::NT, Cfg<N>::PER_256 * BPS_XLEAP_MIN_BLOCKS)
     k_xleap_wring(Fields fp0, XArgs xa, const __grid_constant__ XMaps maps) {
   using XR = XRing<N>;
   const Fields fp = at_chain(fp0, blockIdx.y);
@@ -1941,7 +1941,7 @@ bool make_xmaps(const Fields& f, int N, int nch, XMaps* out) {
   }();
   if (!encode) return false;
   const int ZP = ((N / 2 + 1) + 1) / 2 * 2;
-  const int F = N / 2 < 16 ? N / 2 : 16;
+  const int F = N / 2 < 16 ? N / 2 : N == 128 ? 8 : 16;   // Cfg<N>::F
   const unsigned long long plane = (unsigned long long)N * N * ZP;
   const unsigned long long cs = f.spec_stride > 0 ? (unsigned long long)f.spec_stride : plane;
   const cuuint64_t dims[4] = {(cuuint64_t)ZP, (cuuint64_t)N, (cuuint64_t)N, (cuuint64_t)(nch > 0 ? nch : 1)};

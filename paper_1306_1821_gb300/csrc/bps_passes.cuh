@@ -124,7 +124,9 @@ enum { MAP_COL = 0, MAP_ROW = 1 };
 
 template <int MAP, int A, int B, int F>
 __device__ __forceinline__ int exidx(int f, int a, int c) {
-  if constexpr (MAP == MAP_COL) return (c * A + a) * F + f;
+  // eight columns: a half warp reads two values of c, kept on different halves of the banks
+  if constexpr (MAP == MAP_COL && F == 8 && A % 2 == 0) return (c * A + (a ^ (c & 1))) * F + f;
+  else if constexpr (MAP == MAP_COL) return (c * A + a) * F + f;
   else return f * (B * (A + 1)) + c * (A + 1) + a;
 }
 
