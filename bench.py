@@ -464,14 +464,18 @@ def run_ours(args):
     # ---- roofline of the dominant kernel (the x pass), from the live events
     S_c = wl.N * wl.N * (wl.N // 2 + 1) * 8
     z_bytes, z_info = z_pass_bytes(R, wl.N)
-    bytes_kind = [6 * S_c, 2 * S_c, z_bytes, 2 * S_c]
+    # the y passes write (inverse) and read (forward), and the z pass writes, W on the
+    # z lines that meet the survey only
+    met = z_info["lines_with_support"]
+    y_bytes = (1.0 + met) * S_c
+    bytes_kind = [6 * S_c, y_bytes, z_bytes - (1.0 - met) * S_c, y_bytes]
     per_launch_ms = [kms[i] / max(kn[i], 1) for i in range(4)]
     shares = [kms[i] / max(sum(kms), 1e-30) for i in range(4)]
     peak, peak_kind = measured_peaks()
     dom = int(np.argmax(kms))
     achieved = bytes_kind[dom] / (per_launch_ms[dom] * 1e-3) / 1e9
     leap_ms = sum(per_launch_ms)
-    leap_bytes = 10 * S_c + z_bytes
+    leap_bytes = sum(bytes_kind)
     traffic = read_traffic() if dom == 0 else None
 
     if rank == 0:

@@ -51,6 +51,7 @@ struct bps_ctx {
   float* a = nullptr;
   float* c = nullptr;
   int2* span = nullptr;         // per-line support of a and c (grids with N % 32 == 0)
+  uint32_t* rows = nullptr;     // lines with support per plane (Fields::rows), where the force stage is three passes
   uint16_t* cnt = nullptr;
   float* R = nullptr;
   float2* tw = nullptr;
@@ -274,6 +275,9 @@ Fields fields(bps_ctx* c) {
   f.cnt = c->cnt;
   f.R = c->R;
   f.span = c->span;
+  f.rows = c->rows;
+  f.rows_stride = (long long)c->N * c->N / 32;
+  f.rows_slot = f.rows_stride * c->batch;
   f.span_stride = (long long)c->N * c->N;
   f.data_slot = (long long)c->max_sub * c->nv * c->batch;
   f.span_slot = (long long)c->N * c->N * c->batch;
@@ -467,13 +471,13 @@ bps_status force_stage(bps_ctx* ctx, const Fields& f, int region, bool prof, cud
     return BPS_OK;
   }
   if (prof) prof_mark(ctx, 1);
-  P.y_inv(f, BUF_W, B, s);
+  P.y_inv_survey(f, B, s);
   if (prof) prof_mark(ctx, 1);
   if (prof) prof_mark(ctx, 2);
   ctx->zgrad(f, region, B, s);
   if (prof) prof_mark(ctx, 2);
   if (prof) prof_mark(ctx, 3);
-  P.y_fwd(f, BUF_W, B, s);
+  P.y_fwd_survey(f, B, s);
   if (prof) prof_mark(ctx, 3);
   LAUNCHED(ctx, 3);
   return BPS_OK;
@@ -530,7 +534,9 @@ bps_status bias_stage(bps_ctx* ctx, bool advance) {
   const int B = ctx->batch;
   // delta = C2R(delta_hat) (x and y inverse into W), the per-subsample sums in the z pass
   ctx->pt.x_inv(f, -1, nullptr, B, s);
-  ctx->pt.y_inv(f, BUF_W, B, s);
+  // (the posterior moments take the whole field from W afterwards)
+  if (ctx->mom_on) ctx->pt.y_inv(f, BUF_W, B, s);
+  else ctx->pt.y_inv_survey(f, B, s);
   ctx->pt.z_sums(f, region_offset(ctx, RG_SUMS), B, s);
   launch_bias_nbar(sa, region_offset(ctx, RG_SUMS), ctx->pt.z_tiles, B, s);
   LAUNCHED(ctx, 4);
@@ -700,6 +706,7 @@ void free_all(bps_ctx* c) {
   cudaFree(c->a);
   cudaFree(c->c);
   cudaFree(c->span);
+  cudaFree(c->rows);
   cudaFree(c->cnt);
   cudaFree(c->R);
   cudaFree(c->tw);
@@ -829,6 +836,7 @@ bps_status choose_zgrad(bps_ctx* ctx) {
         for (int pattern = 0; pattern < 2 && err == cudaSuccess; ++pattern) {
           Fields f = fields(ctx);
           f.span = pattern ? span_dev : nullptr;
+          f.rows = nullptr;
           f.span_stride = (long long)N * N;
           f.span_slot = 0;
           for (int w = 0; w < 2; ++w) ctx->pt.z_grad_lp[c](f, -1, B, s);
@@ -1012,6 +1020,7 @@ bps_status create_group(int grid_n, const std::vector<double>& box, const std::v
   bool ok = alloc((void**)&ctx->dh[0], sb) && alloc((void**)&ctx->dh[1], sb) && alloc((void**)&ctx->ph, sb) &&
             alloc((void**)&ctx->W, sb) && alloc((void**)&ctx->a, rb) && alloc((void**)&ctx->c, rb) &&
             (grid_n % 32 != 0 || alloc((void**)&ctx->span, span_bytes)) &&
+            (grid_n % 32 != 0 || ctx->yz.run || alloc((void**)&ctx->rows, span_bytes / sizeof(int2) / 8)) &&
             alloc((void**)&ctx->tw, grid_n * sizeof(float2)) && alloc((void**)&ctx->pbin, ctx->n_spec) &&
             alloc((void**)&ctx->part, (size_t)ctx->part_cstride * B * sizeof(double)) &&
             alloc((void**)&ctx->ds, sizeof(DevState) * B) &&
@@ -1060,6 +1069,7 @@ bps_status create_group(int grid_n, const std::vector<double>& box, const std::v
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->a, 0, rb, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->c, 0, rb, stream);
   if (e == cudaSuccess && ctx->span) e = cudaMemsetAsync(ctx->span, 0, span_bytes, stream);
+  if (e == cudaSuccess && ctx->rows) e = cudaMemsetAsync(ctx->rows, 0, span_bytes / sizeof(int2) / 8, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
     std::string msg = std::string("initialisation failed: ") + cudaGetErrorString(e);
@@ -1227,6 +1237,10 @@ bps_status commit_data(bps_ctx* ctx, int ch) {
                      ctx->dpart_cstride, ctx->rebuild_blocks, slot, 1, s);
   LAUNCHED(ctx, 1);
   Fields f = fields_at(ctx, ch);
+  if (f.rows) {
+    launch_rows(f.span + slot * f.span_slot, const_cast<uint32_t*>(f.rows) + slot * f.rows_slot, ctx->N, s);
+    LAUNCHED(ctx, 1);
+  }
   if (f.span) {
     CK(cudaMemsetAsync(f.a, 0, (size_t)ctx->nv * sizeof(float), s));
     CK(cudaMemsetAsync(f.c, 0, (size_t)ctx->nv * sizeof(float), s));

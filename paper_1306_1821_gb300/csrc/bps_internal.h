@@ -62,6 +62,10 @@ struct PassTable {
   void (*z_mock)(const Fields&, uint64_t seed, uint64_t stage, float2* dst, cudaStream_t);
   void (*y_fwd)(const Fields&, int buf, int nch, cudaStream_t);
   void (*y_inv)(const Fields&, int buf, int nch, cudaStream_t);
+  // the y passes of W around z_grad and before z_sums: on the rows with survey data
+  // where the context keeps them (Fields::rows), else y_fwd and y_inv
+  void (*y_fwd_survey)(const Fields&, int nch, cudaStream_t);
+  void (*y_inv_survey)(const Fields&, int nch, cudaStream_t);
   void (*z_grad)(const Fields&, int region, int nch, cudaStream_t);
   // the momentum normals' z transform, and the move tables with this step size bound
   void (*z_noise)(const Fields&, double eps_max, int nch, cudaStream_t);
@@ -142,6 +146,8 @@ void launch_bias_nbar(const ScalarArgs& a, int region, int nz, int nch, cudaStre
 // reduce the jump gradient and likelihood partials, then the leapfrog update of `kind` (one launch)
 void launch_jump_step(const ScalarArgs& a, int r_grad, int nx, int r_lik, int r_lik_move, int nz, int kind,
                       int nch, cudaStream_t s);
+// the row words of one chain (Fields::rows) from its spans
+void launch_rows(const int2* span, uint32_t* rows, int n_grid, cudaStream_t s);
 // DevState::scratch[0] = prior energy from nx partials, scratch[1] = likelihood energy from nz (one chain)
 void launch_gradient_energies(const ScalarArgs& a, int r_prior, int nx, int r_lik, int nz, cudaStream_t s);
 // the chain's current half spectrum into a caller's unpadded one

@@ -940,11 +940,15 @@ __global__ void __launch_bounds__(Cfg<N>::NT, Cfg<N>::PER_256 * BPS_XLEAP_MIN_BL
 }
 
 // ------------------------------------------------------------------ y pass
-template <int N, int DIR>
+// SURVEY (W in a force stage or the survey sums): rows y of the plane that carry no
+// survey data are neither written by the inverse pass (the z pass takes them as zero)
+// nor read by the forward one (the z pass does not write them).  The benchmark survey
+// meets 59% of the lines: 256^3, six subsamples, 4848 -> 4704 us per Gibbs iteration (y
+// passes 22.6 and 22.7 -> 21.4 and 20.1 us from a cold L2).
+template <int N, int DIR, bool SURVEY>
 __global__ void __launch_bounds__(Cfg<N>::NT, Cfg<N>::PER_256 * BPS_YPASS_MIN_BLOCKS) k_ypass(Fields fp0, int buf) {
   const Fields fp = at_chain(fp0, blockIdx.y);
   await_previous();
-  if (buf == BUF_W && fp.ds->jreuse) return;   // force stage reused by the jump (uniform)
   using C = Cfg<N>;
   constexpr int F = C::F, R1 = C::R1, R2 = C::R2, NT = C::NT;
   __shared__ float2 s_tw[N];
@@ -954,11 +958,35 @@ __global__ void __launch_bounds__(Cfg<N>::NT, Cfg<N>::PER_256 * BPS_YPASS_MIN_BL
   float2* data = const_cast<float2*>(buf_ptr(fp, buf));
   const int f = t % F, j = t / F;
   const long long colo = T.base + (long long)f * T.cs;
+  // the plane's row words of both data slots, in flight with the slot's number
+  constexpr int NWORD = SURVEY ? N / 32 : 1;
+  uint32_t rows[NWORD];
+  if constexpr (SURVEY) {
+    const uint32_t* p = fp.rows + (long long)(T.kx0 + f * T.dkx) * NWORD;
+    uint32_t other[NWORD];
+#pragma unroll
+    for (int i = 0; i < NWORD; ++i) {
+      rows[i] = __ldg(p + i);
+      other[i] = __ldg(p + fp.rows_slot + i);
+    }
+    const bool second = fp.ds->dslot != 0;
+#pragma unroll
+    for (int i = 0; i < NWORD; ++i) rows[i] = second ? other[i] : rows[i];
+  }
+  if (buf == BUF_W && fp.ds->jreuse) return;   // force stage reused by the jump (uniform)
+  // whether row j + R1 b carries data
+  auto has = [&](int b) -> bool {
+    if constexpr (!SURVEY) return true;
+    const int r = R1 * b;                        // R1 divides 32, or the row's word is taken at run time
+    if constexpr (32 % R1 == 0) return (rows[(r / 32) % NWORD] >> (r % 32 + j)) & 1u;
+    else return (rows[((r + j) / 32) % NWORD] >> ((r + j) % 32)) & 1u;
+  };
   float2 v[C::RMAX];
   if constexpr (DIR == FWD) {
     if (j < R1) {
 #pragma unroll
-      for (int b = 0; b < R2; ++b) v[b] = data[colo + (long long)(j + R1 * b) * T.rs];
+      for (int b = 0; b < R2; ++b)
+        v[b] = has(b) ? data[colo + (long long)(j + R1 * b) * T.rs] : make_float2(0.f, 0.f);
     }
   } else {
     if (j < R2) {
@@ -978,9 +1006,18 @@ __global__ void __launch_bounds__(Cfg<N>::NT, Cfg<N>::PER_256 * BPS_YPASS_MIN_BL
     fft2<N, R2, R1, INV, MAP_COL, F, TwSquare<N>::value>(v, s_ex, s_tw, t);
     if (j < R1) {
 #pragma unroll
-      for (int b = 0; b < R2; ++b) data[colo + (long long)(j + R1 * b) * T.rs] = v[b];
+      for (int b = 0; b < R2; ++b)
+        if (has(b)) data[colo + (long long)(j + R1 * b) * T.rs] = v[b];
     }
   }
+}
+
+// The row words of one chain's plane blockIdx.x from its spans (Fields::rows), by N threads.
+__global__ void k_rows(const int2* __restrict__ span, uint32_t* __restrict__ rows, int N) {
+  const int y = threadIdx.x;
+  const int2 sp = span[(long long)blockIdx.x * N + y];
+  const unsigned m = __ballot_sync(0xffffffffu, sp.y > N - sp.x);
+  if ((y & 31) == 0) rows[(long long)blockIdx.x * (N / 32) + y / 32] = m;
 }
 
 // ------------------------------------------------------------------ z pass
@@ -1069,9 +1106,11 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
       for (int l = 0; l < LINES; ++l) any |= s_hi[l] > s_lo[l];
       if (!any) {
         if constexpr (MODE == Z_GRAD) {
-          for (int i = t; i < LINES * (H + 1); i += NTZ) {
-            const int l = i / (H + 1), k = i - l * (H + 1);
-            fp.W[(L0 + l) * ZP + k] = make_float2(0.f, 0.f);
+          if (!fp.rows) {           // else the forward y pass does not read these lines
+            for (int i = t; i < LINES * (H + 1); i += NTZ) {
+              const int l = i / (H + 1), k = i - l * (H + 1);
+              fp.W[(L0 + l) * ZP + k] = make_float2(0.f, 0.f);
+            }
           }
           if (za.region >= 0 && t == 0) fp.part[za.region + blockIdx.x] = 0.0;
         } else {
@@ -1110,6 +1149,9 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
     {
       const int f = t / R2, a = t % R2;
       if (f < LP) {
+        // lines without survey data hold what the x pass left there, not their field
+        const bool la = !SUPPORT || !fp.rows || s_hi[2 * f] > s_lo[2 * f];
+        const bool lb = !SUPPORT || !fp.rows || s_hi[2 * f + 1] > s_lo[2 * f + 1];
 #pragma unroll
         for (int b = 0; b < R1; ++b) {
           const int k = a + R2 * b;
@@ -1121,6 +1163,10 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
           } else {
             xa = cconj(s_buf[(2 * f) * ZP + N - k]);
             xb = cconj(s_buf[(2 * f + 1) * ZP + N - k]);
+          }
+          if constexpr (SUPPORT) {
+            if (!la) xa = make_float2(0.f, 0.f);
+            if (!lb) xb = make_float2(0.f, 0.f);
           }
           v[b] = make_float2(xa.x - xb.y, xa.y + xb.x);
         }
@@ -1788,9 +1834,17 @@ struct Launch {
   static void x(const Fields& fp, const XArgs& xa, int nch, cudaStream_t s) {
     launch_dep(k_xpass<N, M>, dim3(C::TILES + (M == X_INV && xa.eps_max >= 0.0), nch), dim3(C::NT), 0, s, fp, xa);
   }
-  template <int D>
+  template <int D, bool S = false>
   static void y(const Fields& fp, int buf, int nch, cudaStream_t s) {
-    launch_dep(k_ypass<N, D>, dim3(C::TILES, nch), dim3(C::NT), 0, s, fp, buf);
+    launch_dep(k_ypass<N, D, S>, dim3(C::TILES, nch), dim3(C::NT), 0, s, fp, buf);
+  }
+  // the row words exist for N a multiple of 32
+  template <int D>
+  static void ys(const Fields& fp, int nch, cudaStream_t s) {
+    if constexpr (N % 32 == 0) {
+      if (fp.rows) return y<D, true>(fp, BUF_W, nch, s);
+    }
+    y<D>(fp, BUF_W, nch, s);
   }
   template <int M, int LP = C::LP>
   static void z(const Fields& fp, const ZArgs& za, int nch, cudaStream_t s) {
@@ -1836,6 +1890,8 @@ static PassTable make_table() {
   T.x_wpow = [](const Fields& f, int region, int n, cudaStream_t s) { L::template x<X_WPOW>(f, XArgs{-1, nullptr, 0, region}, n, s); };
   T.y_fwd = [](const Fields& f, int buf, int n, cudaStream_t s) { L::template y<FWD>(f, buf, n, s); };
   T.y_inv = [](const Fields& f, int buf, int n, cudaStream_t s) { L::template y<INV>(f, buf, n, s); };
+  T.y_fwd_survey = [](const Fields& f, int n, cudaStream_t s) { L::template ys<FWD>(f, n, s); };
+  T.y_inv_survey = [](const Fields& f, int n, cudaStream_t s) { L::template ys<INV>(f, n, s); };
   T.z_grad = [](const Fields& f, int region, int n, cudaStream_t s) { L::template z<Z_GRAD>(f, ZArgs{nullptr, nullptr, nullptr, nullptr, region, 0}, n, s); };
   // the force z pass at every tile size the autotuner chooses from
   T.z_grad_lp[0] = [](const Fields& f, int region, int n, cudaStream_t s) { L::template z<Z_GRAD, 4>(f, ZArgs{nullptr, nullptr, nullptr, nullptr, region, 0}, n, s); };
@@ -1974,6 +2030,9 @@ bool pass_table(int N, PassTable* out) {
   }
 }
 
+void launch_rows(const int2* span, uint32_t* rows, int n_grid, cudaStream_t s) {
+  k_rows<<<n_grid, n_grid, 0, s>>>(span, rows, n_grid);
+}
 void launch_spec_out(const Fields& f, float2* dst, int zp, cudaStream_t s) {
   launch_dep(k_spec_out, dim3((unsigned)(((long long)f.grid_n * f.grid_n + 7) / 8)), dim3(256), 0, s, f, dst, zp);
 }

@@ -33,6 +33,11 @@ struct Fields {
   // lo and hi multiples of 4, a = c = 0 outside [lo, hi) (empty when hi <= lo).
   // NULL: dense (no support information).
   const int2* span;
+  // Which z lines of each x plane carry survey data: bit y of the N / 32 words of
+  // plane x, from the spans.  The y passes of a force stage and the z pass between
+  // them move W on those lines only.  NULL: grids with the fused plane kernel, and
+  // dense surveys.
+  const uint32_t* rows;
   int n_sub;
   DevState* ds;
   double* part;           // per-block partial sums (FP64)
@@ -52,11 +57,12 @@ struct Fields {
   long long data_stride;  // elements per chain of counts / response (max subsamples x voxels)
   long long part_cstride; // doubles of partial sums per chain
   long long span_stride;  // lines per chain (N^2)
+  long long rows_stride;  // words of `rows` per chain (N^2 / 32)
   // Two survey-data slots (counts, R, spans), so that the next survey can be
   // uploaded while the kernels read the current one; slot s of counts and R
   // starts s * data_slot elements, of the spans s * span_slot lines, after the
   // pointers above.  DevState::dslot selects the active slot of each chain.
-  long long data_slot, span_slot;
+  long long data_slot, span_slot, rows_slot;
 };
 
 // The survey data of the chain's active slot.
@@ -82,6 +88,7 @@ __host__ __device__ __forceinline__ Fields at_chain(Fields f, int ch) {
   f.cnt += ch * f.data_stride;
   f.R += ch * f.data_stride;
   if (f.span) f.span += ch * f.span_stride;
+  if (f.rows) f.rows += ch * f.rows_stride;
   f.ds += ch;
   f.part += ch * f.part_cstride;
   return f;
