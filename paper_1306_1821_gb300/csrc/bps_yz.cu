@@ -17,7 +17,8 @@
 //     transform) from C2R through the local force to R2C: the exchanges go through
 //     the pair's own two rows with warp barriers only, and a warp whose lines
 //     carry no survey data writes zeros.
-// Rows are SP = ZP + 1 (odd) complex apart and the exchange within a pair is
+// Rows are SP = N/2 + 1 (odd) complex apart, so that consecutive tasks of a first y half
+// touch consecutive elements across rows, and the exchange within a pair is
 // swizzled (zpos), which keeps the 8-byte accesses of a half warp on distinct banks.
 //
 // Measured per launch under ncu against the form with a block-wide exchange buffer
@@ -34,7 +35,7 @@ template <int N, int NWARPS>
 struct YZ {
   static constexpr int B = Cfg<N>::R1, A = Cfg<N>::R2;   // N = B A, B >= A
   static constexpr int ZP = Cfg<N>::ZP, H = N / 2, COLS = H + 1;
-  static constexpr int SP = ZP + 1;                      // row pitch in shared memory (complex)
+  static constexpr int SP = COLS;                        // row pitch in shared memory (complex)
   static constexpr int T1 = A * COLS, T2 = B * COLS;     // tasks of the two halves of a y transform
   static constexpr int PAIRS = 4, LINES = 2 * PAIRS;     // z lines of one warp unit
   static constexpr int UNITS = N / LINES;
