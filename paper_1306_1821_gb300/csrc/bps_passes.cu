@@ -162,6 +162,48 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   if constexpr (MODE == X_JINV) {
     if (ds->jreuse) return;       // W already holds this force stage's input (uniform)
   }
+  const Tile<N> T = tile_x<N>(tile_id<N>());
+  const int f = t % F;
+  const int ja = t / F;                       // row group of the spatial (x-) layout
+  const int ky = T.ky0 + f * T.dky, kz = T.kz0 + f * T.dkz;
+  const int ny = sgn_n<N>(ky);
+  const int n2yz = ny * ny + kz * kz;
+  const float wk = (kz == 0 || kz == C::H) ? 1.f : 2.f;
+  const long long colo = T.base + (long long)f * T.cs;
+  const int cur = ds->cur;
+  const bool mm = fp.mass_mode != 0;
+  const float scb = bin_scale(fp.n_bins, N), scm = bin_scale(fp.n_mass, N);
+
+  float2 v[C::RMAX];
+  // Modes that start from a spatial-x tile send its loads out before the tables below
+  // are read.  Where one grid's tiles are few (up to 96^3) the loads of the column's
+  // other data go with them, so that a block waits for memory once instead of for W
+  // and each part in turn: Gibbs iteration at 32^3 155 -> 145 us, 96^3 move 264 -> 255 us.  At
+  // 128^3 (1040 tiles) the registers cost more than that: 710 -> 720 us.
+  constexpr bool SPATIAL = MODE == X_INIT || MODE == X_LEAP || MODE == X_LEAPG || MODE == X_FINAL || MODE == X_FWD ||
+                           MODE == X_GRAD || MODE == X_JGRAD || MODE == X_AMP;
+  constexpr bool KICK = MODE == X_LEAP || MODE == X_LEAPG || MODE == X_FINAL;
+  constexpr bool EARLY = N <= 96 && (KICK || MODE == X_INIT || MODE == X_GRAD);
+  float2 ex[EARLY ? R1 : 1], ep[EARLY && KICK ? R1 : 1];
+  if constexpr (SPATIAL) {
+    const float2* in = (MODE == X_INIT) ? fp.ph : (MODE == X_FWD) ? buf_ptr(fp, xa.src_buf) : fp.W;
+    // X_FWD with no destination writes the current state buffer
+    if (ja < R1) {
+#pragma unroll
+      for (int b = 0; b < R2; ++b) v[b] = in[colo + (long long)(ja + R1 * b) * T.rs];
+    }
+  }
+  if constexpr (EARLY) {
+    const float2* src = dsel(fp, MODE == X_FINAL || (MODE == X_LEAP && !xa.first) ? 1 - cur : cur);
+    if (ja < R2) {
+#pragma unroll
+      for (int d = 0; d < R1; ++d) {
+        const long long idx = colo + (long long)(ja + R2 * d) * T.rs;
+        ex[d] = src[idx];
+        if constexpr (KICK) ep[d] = fp.ph[idx];
+      }
+    }
+  }
   for (int i = t; i < MAXB; i += NT) {
     s_thr[i] = ds->thr[i];
     s_mthr[i] = ds->mthr[i];
@@ -180,24 +222,11 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   }
   __syncthreads();
 
-  const Tile<N> T = tile_x<N>(tile_id<N>());
-  const int f = t % F;
-  const int ja = t / F;                       // row group of the spatial (x-) layout
-  const int ky = T.ky0 + f * T.dky, kz = T.kz0 + f * T.dkz;
-  const int ny = sgn_n<N>(ky);
-  const int n2yz = ny * ny + kz * kz;
-  const float wk = (kz == 0 || kz == C::H) ? 1.f : 2.f;
-  const long long colo = T.base + (long long)f * T.cs;
-  const int cur = ds->cur;
-  const bool mm = fp.mass_mode != 0;
-  const float scb = bin_scale(fp.n_bins, N), scm = bin_scale(fp.n_mass, N);
-
-  float2 v[C::RMAX];
   // modes that update or reduce the column against delta and p work through it in
   // parts: the loads of a part in flight together, at a fraction of the registers
   // of a whole column
   constexpr bool WHOLE = (MODE == X_INIT || MODE == X_FINAL || MODE == X_GRAD) && !XParts<N>::value;
-  constexpr int PART = WHOLE ? R1 : R1 / BPS_XLEAP_CHUNKS > 0 ? R1 / BPS_XLEAP_CHUNKS : 1;
+  constexpr int PART = WHOLE || EARLY ? R1 : R1 / BPS_XLEAP_CHUNKS > 0 ? R1 / BPS_XLEAP_CHUNKS : 1;
   auto mode_bin = [&](int k, float& il, float& im, float& sm) -> int {
     const int nx = sgn_n<N>(k);
     const int n2 = nx * nx + n2yz;
@@ -218,16 +247,7 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
   };
 
   // ---------------- modes that start from a spatial-x tile: forward transform
-  if constexpr (MODE == X_INIT || MODE == X_LEAP || MODE == X_LEAPG || MODE == X_FINAL || MODE == X_FWD ||
-                MODE == X_GRAD || MODE == X_JGRAD || MODE == X_AMP) {
-    const float2* in = (MODE == X_INIT) ? fp.ph : (MODE == X_FWD) ? buf_ptr(fp, xa.src_buf) : fp.W;
-    // X_FWD with no destination writes the current state buffer
-    if (ja < R1) {
-#pragma unroll
-      for (int b = 0; b < R2; ++b) v[b] = in[colo + (long long)(ja + R1 * b) * T.rs];
-    }
-    fft2<N, R1, R2, FWD, MAP_COL, F, TwSquare<N>::value>(v, s_ex, s_tw, t);
-  }
+  if constexpr (SPATIAL) fft2<N, R1, R2, FWD, MAP_COL, F, TwSquare<N>::value>(v, s_ex, s_tw, t);
   const int jc = t / F;                       // row group of the Fourier (kx-) layout
   const bool act = jc < R2;
 
@@ -253,7 +273,8 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
       for (int h = 0; h < R1; h += PART) {
         float2 x[PART];
 #pragma unroll
-        for (int q = 0; q < PART; ++q) x[q] = dsel(fp, cur)[colo + (long long)(jc + R2 * (h + q)) * T.rs];
+        for (int q = 0; q < PART; ++q)
+          x[q] = EARLY ? ex[EARLY ? q : 0] : dsel(fp, cur)[colo + (long long)(jc + R2 * (h + q)) * T.rs];
 #pragma unroll
         for (int q = 0; q < PART; ++q) {
           const int d = h + q, k = jc + R2 * d;
@@ -297,8 +318,8 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
 #pragma unroll
       for (int q = 0; q < PART; ++q) {
         const long long idx = colo + (long long)(jc + R2 * (h + q)) * T.rs;
-        x[q] = src[idx];
-        p[q] = fp.ph[idx];
+        x[q] = EARLY ? ex[EARLY ? q : 0] : src[idx];
+        p[q] = EARLY ? ep[EARLY ? q : 0] : fp.ph[idx];
       }
 #pragma unroll
       for (int q = 0; q < PART; ++q) {
@@ -354,8 +375,8 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
 #pragma unroll
         for (int q = 0; q < PART; ++q) {
           const long long idx = colo + (long long)(jc + R2 * (h + q)) * T.rs;
-          x[q] = src[idx];
-          p[q] = fp.ph[idx];
+          x[q] = EARLY ? ex[EARLY ? q : 0] : src[idx];
+          p[q] = EARLY ? ep[EARLY ? q : 0] : fp.ph[idx];
         }
 #pragma unroll
         for (int q = 0; q < PART; ++q) {
@@ -393,7 +414,8 @@ __global__ void __launch_bounds__(Cfg<N>::NT, MODE == X_LEAP || MODE == X_LEAPG 
       for (int h = 0; h < R1; h += PART) {
         float2 x[PART];
 #pragma unroll
-        for (int q = 0; q < PART; ++q) x[q] = dsel(fp, cur)[colo + (long long)(jc + R2 * (h + q)) * T.rs];
+        for (int q = 0; q < PART; ++q)
+          x[q] = EARLY ? ex[EARLY ? q : 0] : dsel(fp, cur)[colo + (long long)(jc + R2 * (h + q)) * T.rs];
 #pragma unroll
         for (int q = 0; q < PART; ++q) {
           const int d = h + q, k = jc + R2 * d;
