@@ -22,8 +22,8 @@
 // swizzled (zpos), which keeps the 8-byte accesses of a half warp on distinct banks.
 //
 // Measured per launch under ncu against the form with a block-wide exchange buffer
-// (256 threads or fewer, 151 registers, 18% of the warp slots): 128^3 20.7 -> 14.4 us;
-// 32 chains of 96^3 162 -> 118 us, of 64^3 54 -> 34 us, of 32^3 10.8 -> 10.4 us.  At 96^3
+// (256 threads or fewer, 151 registers, 18% of the warp slots): 128^3 20.7 -> 13.0 us;
+// 32 chains of 96^3 162 -> 103 us, of 64^3 54 -> 33 us, of 32^3 10.8 -> 9.4 us.  At 96^3
 // the shared-memory pipe is 64-69% busy, with 40% of the warp slots filled.
 #include "bps_internal.h"
 #include "bps_passes.cuh"
