@@ -1317,6 +1317,46 @@ bps_status get_state_chain(bps_ctx* ctx, int ch, float* delta_dev, double* P, do
   return BPS_OK;
 }
 
+// Streams that branch off a capturing stream and join it again before the capture
+// ends; they live for the capture only.
+struct CaptureBranches {
+  std::vector<cudaStream_t> stream;
+  std::vector<cudaEvent_t> done;
+  cudaEvent_t start = nullptr;
+
+  cudaError_t fork(cudaStream_t from, size_t n) {
+    if (n == 0) return cudaSuccess;
+    cudaError_t e = cudaEventCreateWithFlags(&start, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(start, from);
+    for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+      cudaStream_t s = nullptr;
+      cudaEvent_t ev = nullptr;
+      e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+      if (e != cudaSuccess) break;
+      done.push_back(ev);
+      e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+      if (e != cudaSuccess) break;
+      stream.push_back(s);
+      e = cudaStreamWaitEvent(s, start, 0);
+    }
+    return e;
+  }
+  cudaError_t join(cudaStream_t to) {
+    cudaError_t e = cudaSuccess;
+    for (size_t i = 0; i < stream.size(); ++i) {
+      cudaError_t ei = cudaEventRecord(done[i], stream[i]);
+      if (ei == cudaSuccess) ei = cudaStreamWaitEvent(to, done[i], 0);
+      if (e == cudaSuccess) e = ei;
+    }
+    return e;
+  }
+  ~CaptureBranches() {
+    for (cudaStream_t s : stream) cudaStreamDestroy(s);
+    for (cudaEvent_t ev : done) cudaEventDestroy(ev);
+    if (start) cudaEventDestroy(start);
+  }
+};
+
 // Captures one Gibbs iteration of every chain of the groups into *out (kernels
 // counted per replay in *launches).  With `prof` the captured iteration also
 // holds event-record nodes around the leapfrog kernels of top (one group).
@@ -1348,14 +1388,25 @@ bps_status capture_iteration(bps_ctx* top, const std::vector<bps_ctx*>& groups, 
   CK(cudaStreamBeginCapture(top->cap_stream, cudaStreamCaptureModeThreadLocal));
   for (bps_ctx* gr : groups) gr->stream = top->cap_stream;
   top->capturing = prof;
+  // The groups share no buffers (their chains' rows of the record are apart), so each
+  // further group is a branch of the graph: its small kernels and scalar stages run
+  // beside another group's wide passes.  96 chains of 32^3, 64^3 and 96^3: 6900 us per
+  // iteration one group after the other, 6340 as branches (the same with the smaller
+  // groups' streams at a higher priority).  Several groups of one grid size lose more in
+  // smaller launches than they overlap: 6610 us with the 96^3 chains in two, 6450 in four.
+  CaptureBranches br;
   bps_status st = BPS_OK;
-  for (bps_ctx* gr : groups) {
-    st = gibbs_once(gr, rec_dev, rec_len, iter_stride, jump);
-    if (st != BPS_OK) break;
+  cudaError_t e = br.fork(top->cap_stream, groups.size() - 1);
+  for (size_t i = 0; i < groups.size() && e == cudaSuccess && st == BPS_OK; ++i) {
+    if (i) groups[i]->stream = br.stream[i - 1];
+    st = gibbs_once(groups[i], rec_dev, rec_len, iter_stride, jump);
   }
+  const cudaError_t ej = br.join(top->cap_stream);
+  if (e == cudaSuccess) e = ej;
   top->capturing = false;
   for (bps_ctx* gr : groups) gr->stream = s;
-  cudaError_t e = cudaStreamEndCapture(top->cap_stream, &g);
+  const cudaError_t ec = cudaStreamEndCapture(top->cap_stream, &g);
+  if (e == cudaSuccess) e = ec;
   // the kernels were captured, not launched: count them per replay instead
   uint64_t captured = 0;
   for (size_t i = 0; i < groups.size(); ++i) {
@@ -1367,9 +1418,9 @@ bps_status capture_iteration(bps_ctx* top, const std::vector<bps_ctx*>& groups, 
       top->prof_graph_events[k] = top->ev_used[k];
       top->ev_used[k] = 0;
     }
-  if (st != BPS_OK) {
+  if (st != BPS_OK || e != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
-    return st;
+    if (st != BPS_OK) return st;
   }
   CK(e);
   e = cudaGraphInstantiate(out, g, 0);
