@@ -1608,8 +1608,8 @@ __global__ void __launch_bounds__(256) k_rebuild(Fields fp0, long long nv, int r
   if (sd.span) {
     // half a warp per z line, its lanes over the line's support (multiples of 4 voxels,
     // mostly less than 64), the next line's support on its way: a chain of latencies,
-    // 39 us at 256^3 with six subsamples and 73 us for 32 chains of 96^3 with a warp per
-    // line and one load at a time, now 28 and 49 us
+    // under ncu 41 us at 256^3 with six subsamples and 73 us as the mean of three launches for
+    // 32 chains each of 32^3, 64^3 and 96^3 with a warp per line and one load at a time, now 36 and 48 us
     const int n_grid = fp.grid_n;
     const int lines = n_grid * n_grid, gpl = n_grid / 4;   // float4 groups per line
     const int lane = threadIdx.x & 15, step = gridDim.x * 16;
