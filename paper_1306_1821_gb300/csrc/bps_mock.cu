@@ -251,8 +251,9 @@ struct RespArgs {
 // cosine is off by less than 1e-6 and decides the cap outside a margin of 1e-5.
 // Values are computed as FP32 pairs (t = sqrt(S) (n_r - 1) / N, table entries split
 // in two), off by less than 2^-41 of the larger table entry and 2^-43 t of the step
-// between the two, and kept where that cannot change their rounding to FP32; the rest takes the FP64 steps that define
-// the response.  With every voxel in FP64 the kernel was bound by FP64 issue: 2.59
+// between the two (in the segment that holds t: the next one's slope is another),
+// and kept where that cannot change their rounding to FP32; the rest takes the FP64
+// steps that define the response.  With every voxel in FP64 the kernel was bound by FP64 issue: 2.59
 // ms at 256^3 with six subsamples, 0.76 ms with FP64 inside the survey only, now
 // 0.146 ms.
 __device__ __noinline__ float response_exact(const RespArgs& a, int ix, int iy, int iz, double ux, double uy, double uz,
@@ -295,6 +296,8 @@ __global__ void __launch_bounds__(256, 4) k_mock_response(RespArgs a, float2 c2,
   const float uxf = (float)axis[0], uyf = (float)axis[1], uzf = (float)axis[2];
   const float cos_out = (float)a.thr_cos - 1e-5f, cos_in = (float)a.thr_cos + 1e-5f;
   const float jmax = (float)(a.n_r - 2);
+  // the pair and the FP64 t, each within 2^-44 t, may lie on two sides of a radius: undecided
+  const float w_lo = 0x1p-42f * (float)a.n_r, w_hi = 1.f - w_lo;
   const long long nv = (long long)a.N * a.N * a.N;
   const long long i = (blockIdx.x * 256LL + threadIdx.x) * V;
   if (i < nv) {
@@ -326,9 +329,12 @@ __global__ void __launch_bounds__(256, 4) k_mock_response(RespArgs a, float2 c2,
       const float s = sqrtf(Sf);
       const float2 s2 = pair_quick(s, __fdividef(__fmaf_rn(-s, s, Sf), 2.f * s));
       const float2 t = pair_mul(s2, c2);
-      const float j = fminf(fmaxf(floorf(t.x), 0.f), jmax);
+      // the first part may have been rounded up to a radius of the table that t does not reach
+      const float fl = floorf(t.x);
+      const float j = fminf(fmaxf(t.y < 0.f && t.x == fl ? fl - 1.f : fl, 0.f), jmax);
       jt[e] = (int)j;
       w[e] = pair_sum(t.x - j, t.y);   // t.x - j is exact
+      if (w[e].x < w_lo || w[e].x >= w_hi) state[e] = 2;
     }
     for (int l = 0; l < a.n_sub; ++l) {
       float v[V];

@@ -66,3 +66,21 @@ def test_response_at_the_edges_of_the_cap(N, axis, f_sky, offset):
         s.close()
     ref = mock.response(N, box, f_sky, axis, table, box / 2)
     assert np.array_equal(got.view(np.uint32), ref.view(np.uint32))
+
+
+@pytest.mark.parametrize("N,n_r", [(64, 1 << 20), (128, 16385), (256, 4501), (256, 7000), (256, 65537)])
+def test_response_of_rough_tables(N, n_r):
+    """Random tables of many radii: whatever rounding leaves of a voxel's place in the table, the
+    value comes from the segment of the FP64 definition (a neighbouring one gives another slope)."""
+    from paper_1306_1821_gb300 import bps
+    box, axis = 750.0, (0.0, 0.0, 1.0)
+    table = np.random.default_rng(2).uniform(0.0, 1.0, (1, n_r))
+    s = bps.Sampler(N, box, 1, 4)
+    try:
+        R = place(np.zeros(N ** 3, dtype=np.float32), 0)
+        bps.bps_mock_response(s.ctx, 1.0, axis, table, R)
+        got = R.cpu().numpy().reshape(1, N, N, N)
+    finally:
+        s.close()
+    ref = mock.response(N, box, 1.0, axis, table, box / 2)
+    assert np.array_equal(got.view(np.uint32), ref.view(np.uint32)), int((got != ref).sum())
