@@ -289,7 +289,9 @@ __global__ void k_mock_table(RespArgs a, const double* __restrict__ table, long 
   out[i] = make_float2(h, (float)(table[i] - (double)h));
 }
 
-template <int V>
+// EXACT: the FP64 steps for every voxel (boxes whose squared lengths overflow FP64 or
+// lose bits there, which decides the radius cut).
+template <int V, bool EXACT>
 __global__ void __launch_bounds__(256, 4) k_mock_response(RespArgs a, float2 c2, const double* __restrict__ axis,
                                                           const double* __restrict__ table,
                                                           const float2* __restrict__ table2, float* __restrict__ R) {
@@ -319,6 +321,11 @@ __global__ void __launch_bounds__(256, 4) k_mock_response(RespArgs a, float2 c2,
       state[e] = 0;
       jt[e] = 0;
       w[e] = make_float2(0.f, 0.f);
+      if constexpr (EXACT) {
+        any = true;
+        state[e] = 2;
+        continue;
+      }
       if (S >= a.N * a.N || cf < cos_out) continue;
       any = true;
       if (!(cf > cos_in)) {
@@ -599,8 +606,14 @@ bps_status mock_response(const MockView& v, double f_sky, const double* axis, in
   // 16-byte stores where R starts on a 16-byte boundary (every subsample then
   // does: N^3 is a multiple of 4); one block per 1024 voxels, so that the
   // hardware's block order balances the observed region
-  if (aligned16(R_dev)) k_mock_response<4><<<(unsigned)((nv / 4 + 255) / 256), 256, 0, v.stream>>>(a, c2, axis_dev, dt, dt2, R_dev);
-  else k_mock_response<1><<<(unsigned)((nv + 255) / 256), 256, 0, v.stream>>>(a, c2, axis_dev, dt, dt2, R_dev);
+  const unsigned blocks = (unsigned)((nv + 255) / 256), blocks4 = (unsigned)((nv / 4 + 255) / 256);
+  cudaStream_t s = v.stream;
+  if (!(v.box > 1e-120 && v.box < 1e120))
+    k_mock_response<1, true><<<blocks, 256, 0, s>>>(a, c2, axis_dev, dt, dt2, R_dev);
+  else if (aligned16(R_dev))
+    k_mock_response<4, false><<<blocks4, 256, 0, s>>>(a, c2, axis_dev, dt, dt2, R_dev);
+  else
+    k_mock_response<1, false><<<blocks, 256, 0, s>>>(a, c2, axis_dev, dt, dt2, R_dev);
   *v.launches += 2;
   if (cudaGetLastError() != cudaSuccess) {
     set_last_error("bps_mock_response: kernel launch failed");

@@ -84,3 +84,22 @@ def test_response_of_rough_tables(N, n_r):
         s.close()
     ref = mock.response(N, box, 1.0, axis, table, box / 2)
     assert np.array_equal(got.view(np.uint32), ref.view(np.uint32)), int((got != ref).sum())
+
+
+@pytest.mark.parametrize("box", [1e160, 1e150, 1e-150, 1e-158, 1e-170])
+def test_response_of_boxes_whose_squares_leave_fp64(box):
+    """Squared distances that overflow, lose bits or vanish in FP64 decide the radius cut of the
+    definition; the kernel follows it there too."""
+    from paper_1306_1821_gb300 import bps
+    N, axis = 32, (0.3, -0.4, 0.87)
+    table = np.random.default_rng(3).uniform(0.5, 1.0, (1, 17))
+    s = bps.Sampler(N, box, 1, 4)
+    try:
+        R = place(np.zeros(N ** 3, dtype=np.float32), 0)
+        bps.bps_mock_response(s.ctx, 0.5, axis, table, R)
+        got = R.cpu().numpy().reshape(1, N, N, N)
+    finally:
+        s.close()
+    with np.errstate(over="ignore", invalid="ignore"):
+        ref = mock.response(N, box, 0.5, axis, table, box / 2)
+    assert np.array_equal(got.view(np.uint32), ref.view(np.uint32)), int((got != ref).sum())
