@@ -68,7 +68,7 @@ def test_response_at_the_edges_of_the_cap(N, axis, f_sky, offset):
     assert np.array_equal(got.view(np.uint32), ref.view(np.uint32))
 
 
-@pytest.mark.parametrize("N,n_r", [(64, 1 << 20), (128, 16385), (256, 4501), (256, 7000), (256, 65537)])
+@pytest.mark.parametrize("N,n_r", [(64, 363), (128, 179), (256, 282), (64, 1 << 20), (128, 16385), (256, 4501), (256, 7000), (256, 65537)])
 def test_response_of_rough_tables(N, n_r):
     """Random tables of many radii: whatever rounding leaves of a voxel's place in the table, the
     value comes from the segment of the FP64 definition (a neighbouring one gives another slope)."""
