@@ -171,14 +171,16 @@ __device__ __noinline__ int poisson_exact(float r, float d, double b, double nba
 // The same count without FP64 where FP32 pairs decide it: one chunk (lambda
 // safely below 32) of ordinary factors.  The pair for 1 + b d is off by less
 // than 2^-43 (1 + |b d|), that for lambda by less than 2^-42 r Nbar (1 + |b d|),
-// which is below 1e-10 for the factors let through.
+// which is below 1e-10 for the factors let through.  |b d| < 1e12 keeps what r Nbar
+// loses below FP32's smallest value (2^-149) as small; b and Nbar have ordinary
+// splits (mock_counts).
 __device__ __noinline__ int poisson_count(float r, float d, float2 b, float2 nb, double b64, double nbar64, long long i,
                                           int l, uint64_t seed) {
   const float q = __fmul_rn(b.x, d);
   const float2 bd = pair_quick(q, __fmaf_rn(b.y, d, __fmaf_rn(b.x, d, -q)));
   const float2 t = pair_add(make_float2(1.f, 0.f), bd);
   const float2 rn = pair_mul(make_float2(r, 0.f), nb);
-  if (r > 0.f && rn.x * (1.f + fabsf(q)) < 400.f) {   // false for NaN
+  if (r > 0.f && fmaxf(rn.x, 4e-10f) * (1.f + fabsf(q)) < 400.f) {   // false for NaN
     if (t.x <= -1e-6f * (1.f + fabsf(q))) return 0;   // lambda = 0
     float2 lam = pair_mul(rn, t);
     if (lam.x < 0.f) lam = make_float2(0.f, 0.f);     // 1 + b d = 0 to within the pair's error
@@ -212,7 +214,8 @@ __device__ __forceinline__ int gauss_count(float r, float d, double b, double nb
 // 36 for seven blocks per SM instead of four (0.45 ms with six or eight): latency.
 // Four voxels per thread hold 124 registers and two blocks per SM (0.92 ms); one
 // response in flight per thread instead of four takes 0.70 ms.
-template <int NOISE>
+// EXACT: the definition at every voxel.
+template <int NOISE, bool EXACT>
 __global__ void __launch_bounds__(256, 7) k_mock_counts(const float* __restrict__ delta, const float* __restrict__ R,
                                                         long long nv, int nsub, MockSub sub, uint64_t seed,
                                                         int32_t* __restrict__ out) {
@@ -230,6 +233,7 @@ __global__ void __launch_bounds__(256, 7) k_mock_counts(const float* __restrict_
       if (l >= nsub) break;
       int c = 0;
       if constexpr (NOISE) c = gauss_count(r[g], d, sub.b[l], sub.nbar[l], i, l, seed);
+      else if constexpr (EXACT) c = poisson_exact(r[g], d, sub.b[l], sub.nbar[l], i, l, seed);
       else if (!(r[g] == 0.f && isfinite(d)))   // lambda = 0 there
         c = poisson_count(r[g], d, sub.b2[l], sub.nbar2[l], sub.b[l], sub.nbar[l], i, l, seed);
       out[l * nv + i] = c;
@@ -538,6 +542,9 @@ bps_status mock_field(const MockView& v, uint64_t seed, const double* P_n2, floa
 bps_status mock_counts(const MockView& v, uint64_t seed, const float* delta_dev, const float* R_dev, const double* b,
                        const double* nbar, int noise, int32_t* counts_dev) {
   MockSub sub{};
+  // whether the FP32 parts of every b and Nbar hold 46 bits, and b delta cannot overflow FP64
+  bool plain = true;
+  auto ordinary = [](double x) { return x == 0.0 || (std::fabs(x) > 1e-20 && std::fabs(x) < 1e20); };
   for (int l = 0; l < v.n_sub; ++l) {
     if (!std::isfinite(b[l]) || !(nbar[l] >= 0.0) || !std::isfinite(nbar[l])) {
       set_last_error("bps_mock_counts: b must be finite and nbar non-negative");
@@ -545,6 +552,7 @@ bps_status mock_counts(const MockView& v, uint64_t seed, const float* delta_dev,
     }
     sub.b[l] = b[l];
     sub.nbar[l] = nbar[l];
+    plain = plain && ordinary(b[l]) && ordinary(nbar[l]);
     auto split = [](double x) {
       const float h = (float)x;
       return make_float2(h, (float)(x - (double)h));
@@ -556,8 +564,8 @@ bps_status mock_counts(const MockView& v, uint64_t seed, const float* delta_dev,
   // one block per 256 voxels: the hardware's block order balances the observed
   // region, which a fixed stride over few blocks leaves to some of them
   const unsigned blocks = (unsigned)((nv + 255) / 256);
-  if (noise == 0) k_mock_counts<0><<<blocks, 256, 0, v.stream>>>(delta_dev, R_dev, nv, v.n_sub, sub, seed, counts_dev);
-  else k_mock_counts<1><<<blocks, 256, 0, v.stream>>>(delta_dev, R_dev, nv, v.n_sub, sub, seed, counts_dev);
+  auto* k = noise ? k_mock_counts<1, false> : plain ? k_mock_counts<0, false> : k_mock_counts<0, true>;
+  k<<<blocks, 256, 0, v.stream>>>(delta_dev, R_dev, nv, v.n_sub, sub, seed, counts_dev);
   *v.launches += 1;
   if (cudaGetLastError() != cudaSuccess) {
     set_last_error("bps_mock_counts: kernel launch failed");

@@ -103,3 +103,31 @@ def test_response_of_boxes_whose_squares_leave_fp64(box):
     with np.errstate(over="ignore", invalid="ignore"):
         ref = mock.response(N, box, 0.5, axis, table, box / 2)
     assert np.array_equal(got.view(np.uint32), ref.view(np.uint32)), int((got != ref).sum())
+
+
+def test_counts_of_factors_far_from_one():
+    """lambda of ordinary size from factors that FP32 cannot hold, and voxels without response whose
+    field overflows: the counts are those of the FP64 definition."""
+    from paper_1306_1821_gb300 import bps
+    N, n_sub = 32, 2
+    nv = N ** 3
+    rng = np.random.default_rng(8)
+    d = rng.uniform(0.0, 1e7, nv).astype(np.float32)
+    d[:2] = [1e20, -1e20]
+    R = np.zeros((n_sub, nv), dtype=np.float32)
+    R[0] = rng.uniform(1e37, 3e38, nv)
+    b, nbar = [1.0, 1e300], [1e-44, 1.0]
+    s = bps.Sampler(N, 500.0, n_sub, 4)
+    try:
+        c = place(np.zeros(n_sub * nv, dtype=np.int32), 0)
+        bps.bps_mock_counts(s.ctx, 7, place(d, 0), place(R, 0), b, nbar, 0, c)
+        got = c.cpu().numpy().reshape(n_sub, nv)
+    finally:
+        s.close()
+    for l in range(n_sub):
+        with np.errstate(invalid="ignore", over="ignore"):
+            lam = mock.mean_counts(d, R[l], b[l], nbar[l])
+        ok = lam <= 4096.0
+        ref = np.full(nv, 65536, dtype=np.int64)
+        ref[ok] = mock.poisson_counts(lam[ok], 7, l, index=np.nonzero(ok)[0])
+        assert np.array_equal(got[l], ref), (l, int((got[l] != ref).sum()))
