@@ -516,7 +516,7 @@ bps_status bps_selftest_wait(bps_ctx* ctx, uint64_t limit_ns);
  * the line supports of a centred ball of radius 0.45 N, and keeps the smallest
  * total; the choice is cached for the process and
  * in the JSON file named by BPS_TUNE_CACHE (default $HOME/.cache/bps_tune.json),
- * so that later contexts and runs reuse it.  BPS_AUTOTUNE=0 keeps 8.  The tile
+ * so that later contexts and runs of a library with the same passes reuse it.  BPS_AUTOTUNE=0 keeps 8.  The tile
  * size changes only the grouping of the likelihood-energy partial sums. */
 int bps_z_line_pairs(const bps_ctx* ctx);
 

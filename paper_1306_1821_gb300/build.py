@@ -3,6 +3,7 @@
 The translation units compile in parallel; the shared library links the
 CUDA runtime dynamically so that it shares the process's runtime with PyTorch.
 """
+import hashlib
 import os
 import subprocess
 import sys
@@ -17,6 +18,17 @@ UNITS = ["bps_passes.cu", "bps_draws.cu", "bps_api.cu", "bps_noalloc.cu", "bps_m
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-Xptxas", "-warn-spills"]
+# what the autotuners time: their cached choices hold for one revision of these
+PASSES = ["bps_passes.cu", "bps_passes.cuh", "bps_common.cuh", "bps_tma.cuh", "bps_internal.h"]
+
+
+def passes_revision(extra=()):
+    """Ten hexadecimal digits that change with the sources and flags of the field passes."""
+    h = hashlib.sha256(" ".join([*ARCH, *FLAGS, *extra]).encode())
+    for name in PASSES:
+        with open(os.path.join(SRC, name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:10]
 
 
 def nvcc():
@@ -40,10 +52,11 @@ def build(verbose=False, extra=()):
     os.makedirs(OUT, exist_ok=True)
     objs = []
     cmds = []
+    rev = "-DBPS_PASSES_REV=r" + passes_revision(extra)
     for u in UNITS:
         o = os.path.join(OUT, u.replace(".cu", ".o"))
         objs.append(o)
-        cmds.append([nvcc(), *ARCH, *FLAGS, *extra, "-I", os.path.join(HERE, "..", "include"), "-c",
+        cmds.append([nvcc(), *ARCH, *FLAGS, *extra, rev, "-I", os.path.join(HERE, "..", "include"), "-c",
                      os.path.join(SRC, u), "-o", o])
     with ThreadPoolExecutor(len(cmds)) as ex:
         list(ex.map(lambda c: _run(c, verbose), cmds))

@@ -725,12 +725,29 @@ void free_all(bps_ctx* c) {
 // buffers (before any data is set: W is scratch) and keeps the fastest; the
 // choice is cached for the process and in a JSON file (BPS_TUNE_CACHE, else
 // $HOME/.cache/bps_tune.json) so later runs reuse it and give the same
-// chains.  BPS_AUTOTUNE=0 keeps 8 line pairs.  The choice changes only the
+// chains; entries of other revisions of the passes (their kernels have other times)
+// are left alone.  BPS_AUTOTUNE=0 keeps 8 line pairs.  The choice changes only the
 // grouping of the likelihood-energy terms into per-block partial sums
 // (compensated FP32 pairs, one FP64 value per block).
 std::mutex g_tune_mu;
 std::map<std::string, int> g_tune;
 bool g_tune_loaded = false;
+
+// "GPU passes=REV N=.. chains=.. what"; REV comes from the build (build.py), a digest
+// of the passes' sources and flags
+#define BPS_STR2(x) #x
+#define BPS_STR(x) BPS_STR2(x)
+#ifndef BPS_PASSES_REV
+#define BPS_PASSES_REV unversioned
+#endif
+std::string tune_key(const bps_ctx* ctx, const char* what) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceProp prop{};
+  cudaGetDeviceProperties(&prop, dev);
+  return std::string(prop.name) + " passes=" BPS_STR(BPS_PASSES_REV) " N=" + std::to_string(ctx->N) +
+         " chains=" + std::to_string(ctx->batch) + " " + what;
+}
 
 std::string tune_path() {
   if (const char* p = std::getenv("BPS_TUNE_CACHE")) return p;
@@ -787,12 +804,7 @@ bps_status choose_zgrad(bps_ctx* ctx) {
   int pick = 1;   // 8 line pairs
   const char* e = std::getenv("BPS_AUTOTUNE");
   if (!(e && std::atoi(e) == 0)) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceProp prop{};
-    cudaGetDeviceProperties(&prop, dev);
-    const std::string key = std::string(prop.name) + " N=" + std::to_string(ctx->N) + " chains=" +
-                            std::to_string(ctx->batch) + " zpairs";
+    const std::string key = tune_key(ctx, "zpairs");
     std::lock_guard<std::mutex> lk(g_tune_mu);
     if (!g_tune_loaded) tune_load();
     auto it = g_tune.find(key);
@@ -888,12 +900,7 @@ bps_status choose_xleap(bps_ctx* ctx) {
   if (!xe && !tune) return BPS_OK;
   if (!make_xmaps(fields(ctx), ctx->N, ctx->batch, &ctx->xmaps)) return BPS_OK;   // no tensor maps: direct
   if (tune) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceProp prop{};
-    cudaGetDeviceProperties(&prop, dev);
-    const std::string key = std::string(prop.name) + " N=" + std::to_string(ctx->N) + " chains=" +
-                            std::to_string(ctx->batch) + " xleap";
+    const std::string key = tune_key(ctx, "xleap");
     std::lock_guard<std::mutex> lk(g_tune_mu);
     if (!g_tune_loaded) tune_load();
     auto it = g_tune.find(key);
