@@ -847,8 +847,9 @@ bps_status choose_zgrad(bps_ctx* ctx) {
         float total = 0.f;
         for (int pattern = 0; pattern < 2 && err == cudaSuccess; ++pattern) {
           Fields f = fields(ctx);
+          // (with row words, where the context keeps them, the z pass masks single lines and
+          // leaves lines without support unwritten; it does not read the words themselves)
           f.span = pattern ? span_dev : nullptr;
-          f.rows = nullptr;
           f.span_stride = (long long)N * N;
           f.span_slot = 0;
           for (int w = 0; w < 2; ++w) ctx->pt.z_grad_lp[c](f, -1, B, s);
