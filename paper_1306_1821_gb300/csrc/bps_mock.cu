@@ -211,7 +211,8 @@ __device__ __forceinline__ int gauss_count(float r, float d, double b, double nb
 // subsamples with every voxel searched in FP64, 1.72 ms with lambda in FP64 and
 // the search in FP32 at the observed voxels only (FP64 pipe 77% busy), and
 // 0.55 ms with lambda in FP32 pairs as well, 0.42 ms with the registers cut from 64 to
-// 36 for seven blocks per SM instead of four (0.45 ms with six or eight): latency.
+// 32 (56 bytes of spills) for seven blocks per SM instead of four (0.45 ms with six or
+// eight): latency.
 // Four voxels per thread hold 124 registers and two blocks per SM (0.92 ms); one
 // response in flight per thread instead of four takes 0.70 ms.
 // EXACT: the definition at every voxel.

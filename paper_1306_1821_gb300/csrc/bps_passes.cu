@@ -88,7 +88,9 @@ __device__ __forceinline__ const float2* buf_ptr(const Fields& fp, int b) {
 #define BPS_XPASS_MIN_BLOCKS 2
 #endif
 // the leapfrog x pass works through its column in BPS_XLEAP_CHUNKS parts, so
-// that BPS_XLEAP_MIN_BLOCKS CTAs of 256 threads fit on an SM without spills
+// that BPS_XLEAP_MIN_BLOCKS CTAs of 256 threads fit on an SM at 80 registers; at 256^3
+// it spills 16 bytes per thread (the first step's form 36, at 96^3 24) since its
+// stores became streaming ones, which gain more (k_xpass)
 #ifndef BPS_XLEAP_MIN_BLOCKS
 #define BPS_XLEAP_MIN_BLOCKS 3
 #endif
@@ -1271,8 +1273,9 @@ __global__ void __launch_bounds__(LP * Cfg<N>::RMAX) k_zpass(Fields fp0, ZArgs z
       // that sixteen lanes share a line's support in 16-byte loads of R and 8-byte
       // loads of the counts, three subsamples' in flight, with the transform's
       // registers free again.  A thread's FP32 sums of its terms (at most 32 for a dense
-      // survey) go to shared memory per quantity, and eight lanes add each quantity's
-      // as compensated pairs: one reduction per tile instead of five shuffle steps per
+      // survey, in chains of at most 10 additions; as far from 64 bits as the chains of up
+      // to 17 of the form before) go to shared memory per quantity, and eight lanes add
+      // each quantity's as compensated pairs: one reduction per tile instead of five shuffle steps per
       // quantity and warp, which were most of this pass's instructions (111 registers,
       // 22% of the warp slots, 84 us at 256^3 with six subsamples, 35 us at 128^3 with
       // fifteen; now 42 and 22 us).

@@ -47,8 +47,9 @@ struct YZ {
   static constexpr size_t OFF_TB = OFF_TA + (size_t)N * sizeof(float2);   // W^(c e) at e B + c
   static constexpr size_t BYTES = OFF_TB + (size_t)N * sizeof(float2);
   static_assert(PAIRS * A <= 32, "a unit's first z half is one round");
-  static_assert(SP % 2 == 1 && UNITS * LINES == N , "layout");
-  // blocks per SM that the registers allow without spills
+  static_assert(SP % 2 == 1 && UNITS * LINES == N, "layout");
+  // blocks per SM that the registers allow with at most 12 bytes of spills (the narrow block at
+  // 64^3, capped at 72 registers; the others have none)
   static constexpr int MIN_BLOCKS = 65536 / (NT * (N == 96 ? 73 : 80)) > 0 ? 65536 / (NT * (N == 96 ? 73 : 80)) : 1;
 };
 
